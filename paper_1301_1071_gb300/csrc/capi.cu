@@ -38,8 +38,6 @@ cudaError_t launch_rowmul_f64(const KernelCfg&, const void*, const double*, cons
                               int, int64_t, int64_t, void*, int32_t*, cudaStream_t);
 cudaError_t launch_rowmul_f32(const KernelCfg&, const void*, const double*, const void*, const double*, int64_t,
                               int, int64_t, int64_t, void*, int32_t*, cudaStream_t);
-cudaError_t launch_gram_f64(const void*, const void*, int64_t, int, int, int, int, int, bool, double*, int32_t*,
-                            cudaStream_t);
 cudaError_t launch_gram_f32(const void*, const void*, int64_t, int, int, int, int, int, bool, double*, int32_t*,
                             cudaStream_t);
 
@@ -51,13 +49,15 @@ cudaError_t launch_rowmul(const KernelCfg& k, const void* X, const double* M1, c
 }
 
 cudaError_t launch_gram(int esz, const void* X, const void* Y, int64_t m, int n, double* part, double* G,
-                        int32_t* status, cudaStream_t st, bool acc_storage) {
+                        int32_t* status, cudaStream_t st, bool acc_storage, int* colexp) {
   const GramGeom g = gram_geom(m, n, esz);
-  cudaError_t e =
-      esz == 8 ? launch_gram_f64(X, Y, m, n, g.chunk, g.grid, g.nt, g.tile, acc_storage, part, status, st)
+  int parts = g.grid;
+  const cudaError_t e =
+      esz == 8 ? launch_gram_split(static_cast<const double*>(X), static_cast<const double*>(Y), m, n, g.grid, &parts,
+                                   part, colexp, st)
                : launch_gram_f32(X, Y, m, n, g.chunk, g.grid, g.nt, g.tile, acc_storage, part, status, st);
   if (e != cudaSuccess) return e;
-  return launch_gram_reduce(part, g.grid, n, G, status, st);
+  return launch_gram_reduce(part, parts, n, G, status, st);
 }
 
 cudaError_t launch_local_qr(const KernelCfg& k, const void* A, int64_t m, int n, int64_t b, int64_t bt, int kt,
@@ -85,7 +85,7 @@ cudaError_t launch_local_qr_step1(const Plan& P, const void* A, int64_t m, int64
                                   double* Rst, double* Tst, int32_t* status, cudaStream_t st) {
   const Level& l0 = P.levels[0];
   const int n = static_cast<int>(P.n);
-  if (!P.gram_oz) return launch_local_qr(P.cfg0, A, m, n, b, l0.bt, l0.kt, p, Y, Rst, Tst, status, st);
+  if (!P.gram_split) return launch_local_qr(P.cfg0, A, m, n, b, l0.bt, l0.kt, p, Y, Rst, Tst, status, st);
   return launch_local_qr_nogram_f64(P.cfg0, A, m, n, b, l0.bt, l0.kt, p, Y, Rst, Tst, status, st);
 }
 
@@ -94,8 +94,8 @@ cudaError_t launch_step1(const Plan& P, const void* A, int64_t m, int64_t b, int
   const Level& l0 = P.levels[0];
   const int n = static_cast<int>(P.n);
   cudaError_t e = launch_local_qr_step1(P, A, m, b, p, Y, Rst, Tst, status, st);
-  if (e != cudaSuccess || !P.gram_oz) return e;
-  return launch_gram_oz(static_cast<const double*>(Y), m, n, b, P.cfg0.B, l0.bt, l0.kt, p, Tst, status, st);
+  if (e != cudaSuccess || !P.gram_split) return e;
+  return launch_gram_t_split(static_cast<const double*>(Y), m, n, b, P.cfg0.B, l0.bt, l0.kt, p, Tst, st);
 }
 
 cudaError_t launch_form_q(const KernelCfg& k, const void* Y, int64_t m, int n, int64_t b, int64_t bt, int kt,
@@ -276,9 +276,10 @@ tsqr_status run_tree(const Plan& P, double* R, int64_t ldr, void* work, cudaStre
                                 : launch_local_qr(P.cfg64, S(l - 1), lv.rows, n, lv.b, lv.bt, lv.kt, lv.p, S(l - 1),
                                                   S(l), T(l), status, st);
     if (e != cudaSuccess) return TSQR_ERR_CUDA;
-    if (launch_build_t(T(l), lv.p * lv.kt, n, false, st) != cudaSuccess) return TSQR_ERR_CUDA;
+    const SignFix sf = P.fuse_sign && l == L - 1 ? SignFix{S(L - 1), R, ldr, ctop, status} : SignFix();
+    if (launch_build_t(T(l), lv.p * lv.kt, n, false, st, sf) != cudaSuccess) return TSQR_ERR_CUDA;
   }
-  if (launch_sign_fix(S(L - 1), n, R, ldr, ctop, status, st) != cudaSuccess) return TSQR_ERR_CUDA;
+  if (!P.fuse_sign && launch_sign_fix(S(L - 1), n, R, ldr, ctop, status, st) != cudaSuccess) return TSQR_ERR_CUDA;
   if (extra(ctop, st) != TSQR_OK) return TSQR_ERR_CUDA;
   for (size_t l = L - 1; l >= 1; --l) {
     const Level& lv = P.levels[l];
@@ -309,8 +310,8 @@ tsqr_status run_direct(const Plan& P, const void* A, void* Q, double* R, int64_t
   if (mark(o, 1, st) != TSQR_OK) return TSQR_ERR_CUDA;
   // the T factors' Gram entries on the tensor cores (Ozaki form); like the T
   // build below, it is part of the Step-2 interval of the stage events
-  if (P.gram_oz && launch_gram_oz(static_cast<const double*>(Q), P.m, n, l0.b, P.cfg0.B, l0.bt, l0.kt, l0.p, T(0),
-                                  status, st) != cudaSuccess)
+  if (P.gram_split && launch_gram_t_split(static_cast<const double*>(Q), P.m, n, l0.b, P.cfg0.B, l0.bt, l0.kt, l0.p,
+                                          T(0), st) != cudaSuccess)
     return TSQR_ERR_CUDA;
   // The row blocks' T factors are read only by Step 3 and the tree reads only
   // the stack of R factors, so for a large T build the tree runs on a side
@@ -320,14 +321,16 @@ tsqr_status run_direct(const Plan& P, const void* A, void* Q, double* R, int64_t
   // waits for both.  Small builds stay in line: they take less time than the
   // side stream's set-up is worth (and no workspace of tsqr_direct_static, at
   // most TSQR_STATIC_WORK_BYTES, reaches the threshold).
-  const bool overlap_t = static_cast<size_t>(l0.p) * l0.kt * n * n * sizeof(double) >= kOverlapTBytes;
+  // One row block: no tree to overlap.
+  const bool overlap_t = L > 1 && static_cast<size_t>(l0.p) * l0.kt * n * n * sizeof(double) >= kOverlapTBytes;
   SideStream side;  // on every exit after a fork, `st` is made to wait for the side stream
   cudaStream_t tree_st = st;
   if (overlap_t) {
     if (!side.make(st)) return TSQR_ERR_CUDA;
     tree_st = side.s;
   }
-  if (launch_build_t(T(0), l0.p * l0.kt, n, P.esz == 4, st) != cudaSuccess) return TSQR_ERR_CUDA;
+  const SignFix sf0 = P.fuse_sign && L == 1 ? SignFix{S(0), R, ldr, ctop, status} : SignFix();
+  if (launch_build_t(T(0), l0.p * l0.kt, n, P.esz == 4, st, sf0) != cudaSuccess) return TSQR_ERR_CUDA;
   TSQR_TRY(run_tree(P, R, ldr, work, tree_st, extra));
   TSQR_CUDA(side.rejoin());
   // Step 3: Q_i = Q1_i Q2_i over the Y_i held in Q.
@@ -335,8 +338,8 @@ tsqr_status run_direct(const Plan& P, const void* A, void* Q, double* R, int64_t
   double* C0 = (L == 1) ? ctop : S(0);
   const int64_t cb0 = (L == 1) ? 1 : l0.p;
   const cudaError_t e3 =
-      P.oz3   ? launch_form_q_oz(static_cast<double*>(Q), P.m, n, l0.b, P.cfg0.B, l0.bt, l0.kt, l0.p, T(0), C0, cb0,
-                                 status, st)
+      P.split3 ? launch_form_q_split(static_cast<double*>(Q), P.m, n, l0.b, P.cfg0.B, l0.bt, l0.kt, l0.p, T(0), C0, cb0,
+                                     status, st)
       : P.tc3 ? launch_form_q_tc(static_cast<float*>(Q), P.m, n, l0.b, P.cfg0.B, l0.bt, l0.kt, l0.p, T(0), C0, cb0,
                                  status, st)
               : launch_form_q(P.cfg0, Q, P.m, n, l0.b, l0.bt, l0.kt, l0.p, T(0), C0, cb0, Q, status, st);
@@ -373,8 +376,26 @@ tsqr_status run_r_only(const Plan& P, int esz, const void* X, double* R, void* w
 
 // out = X M1 (+ Y M2): one input over the row blocks of the Step-1
 // configuration; two inputs with the tile sized for two staged inputs.
+// binary64 data with n <= kRowSplitMaxN: the digit products, one pass per input
+// (xsrc / xexp: the scale of X's columns; Y's are orthonormal columns, their
+// own scale).  `out` may be one of the inputs: that one is then taken first,
+// while it is intact.
 tsqr_status rowmul(const Plan& P, const void* X, const double* M1, const void* Y, const double* M2, void* out,
-                   int32_t* status, cudaStream_t st) {
+                   int32_t* status, cudaStream_t st, const double* xsrc = nullptr, const int* xexp = nullptr) {
+  const int ni = static_cast<int>(P.n);
+  if (P.esz == 8 && ni <= kRowSplitMaxN) {
+    const size_t bytes = static_cast<size_t>(P.m) * P.n * 8;
+    auto clash = [&](const void* in) { return in && in != out && overlaps(in, bytes, out, bytes); };
+    if (!clash(X) && !clash(Y) && !(X == out && Y == out)) {
+      const double *x = static_cast<const double*>(X), *y = static_cast<const double*>(Y);
+      double* o = static_cast<double*>(out);
+      const bool y_first = Y && Y == out;
+      if (y_first) TSQR_CUDA(launch_rowmul_split(y, M2, nullptr, nullptr, P.m, ni, false, o, status, st));
+      if (x) TSQR_CUDA(launch_rowmul_split(x, M1, xsrc, xexp, P.m, ni, y_first, o, status, st));
+      if (y && !y_first) TSQR_CUDA(launch_rowmul_split(y, M2, nullptr, nullptr, P.m, ni, x != nullptr, o, status, st));
+      return TSQR_OK;
+    }
+  }
   const bool two = X && Y;
   const KernelCfg& k = two ? P.cfg_rm2 : P.cfg0;
   const int64_t b = two ? P.b_rm2 : P.cfg0.rm_rows;
@@ -471,7 +492,8 @@ tsqr_status run_direct_host(const Plan& P, int chunks, const char* A, char* Qh, 
     TSQR_CUDA(cudaStreamWaitEvent(st, ev_in[c], 0));
     TSQR_CUDA(launch_step1(P, dbuf + r0 * row_bytes, rows, l0.b, pcnt, dbuf + r0 * row_bytes, S0 + b0 * nn,
                            T0 + b0 * l0.kt * nn, status, st));
-    TSQR_CUDA(launch_build_t(T0 + b0 * l0.kt * nn, pcnt * l0.kt, n, P.esz == 4, st));
+    const SignFix sf0 = P.fuse_sign && L == 1 ? SignFix{S0, Rd, n, ctop, status} : SignFix();  // one block, one chunk
+    TSQR_CUDA(launch_build_t(T0 + b0 * l0.kt * nn, pcnt * l0.kt, n, P.esz == 4, st, sf0));
   }
   // Step 2, then R back to the host
   TSQR_TRY(run_tree(P, Rd, n, work, st, [](double*, cudaStream_t) { return TSQR_OK; }));
@@ -485,8 +507,8 @@ tsqr_status run_direct_host(const Plan& P, int chunks, const char* A, char* Qh, 
     double* Cc = (L == 1) ? C0 : C0 + b0 * nn;
     const int64_t cb = (L == 1) ? 1 : pcnt;
     char* Y = dbuf + r0 * row_bytes;
-    TSQR_CUDA(P.oz3   ? launch_form_q_oz(reinterpret_cast<double*>(Y), rows, n, l0.b, P.cfg0.B, l0.bt, l0.kt, pcnt,
-                                         T0 + b0 * l0.kt * nn, Cc, cb, status, st)
+    TSQR_CUDA(P.split3 ? launch_form_q_split(reinterpret_cast<double*>(Y), rows, n, l0.b, P.cfg0.B, l0.bt, l0.kt,
+                                             pcnt, T0 + b0 * l0.kt * nn, Cc, cb, status, st)
               : P.tc3 ? launch_form_q_tc(reinterpret_cast<float*>(Y), rows, n, l0.b, P.cfg0.B, l0.bt, l0.kt, pcnt,
                                          T0 + b0 * l0.kt * nn, Cc, cb, status, st)
                       : launch_form_q(P.cfg0, Y, rows, n, l0.b, l0.bt, l0.kt, pcnt, T0 + b0 * l0.kt * nn, Cc, cb, Y,
@@ -555,15 +577,17 @@ tsqr_status tsqr_launch_count(int32_t op, int64_t m, int64_t n, int32_t dtype, c
                            device_sms());
   if (rc != TSQR_OK) return static_cast<tsqr_status>(rc);
   const int L = static_cast<int>(P.levels.size());
-  const int g = P.gram_oz ? 1 : 0;                     // the tensor-core Gram after Step 1
+  const int g = P.gram_split ? 1 : 0;               // the T factors' Gram after Step 1
+  const int s1 = P.fuse_sign ? 0 : 1;               // the sign fix, where it is a launch of its own
   const int w = (P.tc3 && P.n <= kTcMaxN) ? 1 : 0;  // the W chain before the 3xTF32 chunk stream
   switch (op) {
-    case TSQR_OP_DIRECT_HOST: *launches = (3 + g + w) * chunks + 3 * (L - 1) + 1; break;  // chunks x (Step 1, T, Step 3)
-    case TSQR_OP_DIRECT: *launches = 3 * L + 1 + g + w; break;    // L up (+ T build), sign fix, L down
-    case TSQR_OP_SVD: *launches = 3 * L + 2 + g + w; break;       // + Jacobi SVD
+    case TSQR_OP_DIRECT_HOST: *launches = (3 + g + w) * chunks + 3 * (L - 1) + s1; break;  // chunks x (Step 1, T, Step 3)
+    case TSQR_OP_DIRECT: *launches = 3 * L + s1 + g + w; break;   // L up (+ T build), sign fix, L down
+    case TSQR_OP_SVD: *launches = 3 * L + 1 + s1 + g + w; break;  // + Jacobi SVD
     case TSQR_OP_CHOLQR: *launches = 4 * (1 + refine_steps) + refine_steps; break;  // gram, reduce, chol, rowmul (+ combine)
     case TSQR_OP_INDIRECT: *launches = (L + 3) * (1 + refine_steps) + refine_steps; break;
-    case TSQR_OP_BACKWARD: *launches = 4; break;              // gram, reduce, prep, rowmul
+    // gram, reduce, prep, rowmul (binary64, n <= kRowSplitMaxN: one pass per input)
+    case TSQR_OP_BACKWARD: *launches = P.esz == 8 && P.n <= kRowSplitMaxN ? 5 : 4; break;
     case TSQR_OP_R: *launches = L + 1; break;                 // L levels up (R only), sign fix
     case TSQR_OP_SVD_VALUES: *launches = L + 2; break;        // + Jacobi SVD
     default: return TSQR_ERR_ARG;
@@ -762,11 +786,11 @@ tsqr_status cholqr(const void* A, int64_t m, int64_t n, int64_t lda, int32_t dty
   // Sec. II-A: A^T A = sum_p A_p^T A_p, Cholesky, then Q = A R^{-1} (Sec. II-C)
   TSQR_CUDA(launch_gram(esz, A, A, m, ni, part, G, status, st));
   TSQR_CUDA(launch_chol_inv(G, ni, R1, Rinv, status, st));
-  TSQR_TRY(rowmul(P, A, Rinv, nullptr, nullptr, Q, status, st));
+  TSQR_TRY(rowmul(P, A, Rinv, nullptr, nullptr, Q, status, st, R1));
   for (int r = 0; r < refine_steps; ++r) {  // iterative refinement: repeat on the computed Q
     TSQR_CUDA(launch_gram(esz, Q, Q, m, ni, part, G, status, st));
     TSQR_CUDA(launch_chol_inv(G, ni, R2, Rinv, status, st));
-    TSQR_TRY(rowmul(P, Q, Rinv, nullptr, nullptr, Q, status, st));
+    TSQR_TRY(rowmul(P, Q, Rinv, nullptr, nullptr, Q, status, st, R2));
     TSQR_CUDA(launch_tri_mul(R2, R1, ni, R1, n, st));
   }
   TSQR_TRY(copy_r(R, ldr, R1, n, st));
@@ -795,11 +819,11 @@ tsqr_status tsqr_indirect_refine(const void* A, int64_t m, int64_t n, int64_t ld
   // Sec. II-B: R from the TSQR reduction; Sec. II-C: Q = A R^{-1}
   TSQR_TRY(run_r_only(P, esz, A, R1, work, st));
   TSQR_CUDA(launch_rinv(R1, n, ni, Rinv, status, st));
-  TSQR_TRY(rowmul(P, A, Rinv, nullptr, nullptr, Q, status, st));
+  TSQR_TRY(rowmul(P, A, Rinv, nullptr, nullptr, Q, status, st, R1));
   for (int r = 0; r < refine_steps; ++r) {  // refinement: repeat on the computed Q
     TSQR_TRY(run_r_only(P, esz, Q, R2, work, st));
     TSQR_CUDA(launch_rinv(R2, n, ni, Rinv, status, st));
-    TSQR_TRY(rowmul(P, Q, Rinv, nullptr, nullptr, Q, status, st));
+    TSQR_TRY(rowmul(P, Q, Rinv, nullptr, nullptr, Q, status, st, R2));
     TSQR_CUDA(launch_tri_mul(R2, R1, ni, R1, n, st));
   }
   TSQR_TRY(copy_r(R, ldr, R1, n, st));
@@ -840,10 +864,13 @@ tsqr_status tsqr_backward(const void* Q, const double* R, const void* dQ, const 
   double* M2 = G + 2 * nn;
   const int ni = static_cast<int>(n);
   TSQR_CUDA(cudaMemsetAsync(status, 0, sizeof(int32_t), st));
-  if (dQ) TSQR_CUDA(launch_gram(esz, dQ, Q, m, ni, part, G, status, st, esz == 4));  // G = dQ^T Q
+  // G = dQ^T Q; binary64: with the scale of dQ's columns, for the product below
+  int* qexp = esz == 8 && dQ ? reinterpret_cast<int*>(G + 3 * nn) : nullptr;
+  if (qexp) TSQR_CUDA(cudaMemsetAsync(qexp, 0, n * sizeof(int), st));
+  if (dQ) TSQR_CUDA(launch_gram(esz, dQ, Q, m, ni, part, G, status, st, esz == 4, qexp));
   TSQR_CUDA(launch_bwd_prep(R, dR, dQ ? G : nullptr, ni, M1, M2, status, st));
   // dA = (dQ + Q copyltu(M)) R^{-T} = dQ R^{-T} + Q (copyltu(M) R^{-T})
-  TSQR_TRY(rowmul(P, dQ, M1, Q, M2, dA, status, st));
+  TSQR_TRY(rowmul(P, dQ, M1, Q, M2, dA, status, st, nullptr, qexp));
   return finish(work, opts, st);
 }
 

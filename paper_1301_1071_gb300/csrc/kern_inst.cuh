@@ -170,6 +170,7 @@ cudaError_t TSQR_ROWMUL_NAME(const KernelCfg& k, const void* X, const double* M1
   }
 }
 
+#ifdef TSQR_GRAM_NAME
 // acc_storage: accumulate each CTA's partial Gram in the storage type (the
 // adjoint of binary32 data); else in binary64.
 cudaError_t TSQR_GRAM_NAME(const void* X, const void* Y, int64_t m, int n, int chunk, int grid, int nt, int tile,
@@ -184,6 +185,7 @@ cudaError_t TSQR_GRAM_NAME(const void* X, const void* Y, int64_t m, int n, int c
   return cudaGetLastError();
 }
 
+#endif  // TSQR_GRAM_NAME
 #endif  // TSQR_ROWMUL_NAME
 
 }  // namespace tsqr

@@ -67,9 +67,29 @@ cudaError_t launch_rowmul(const KernelCfg& k, const void* X, const double* M1, c
                           cudaStream_t st);
 // Partial Grams X^T Y (grid partials of n x n binary64), then their fixed-order sum into G.
 // acc_storage: per-CTA partial Grams accumulate in the storage type (binary32
-// data: the FMA pipe); the cross-CTA sum is always binary64.
+// data: the FMA pipe); the cross-CTA sum is always binary64.  binary64 data:
+// launch_gram_split (colexp passed to it).
 cudaError_t launch_gram(int esz, const void* X, const void* Y, int64_t m, int n, double* part, double* G,
-                        int32_t* status, cudaStream_t st, bool acc_storage = false);
+                        int32_t* status, cudaStream_t st, bool acc_storage = false, int* colexp = nullptr);
+
+// binary64 as exact digit products (split_kernels.cuh).  out (+)= X M, n <=
+// kRsMaxN: colsrc / colexp give the scale of X's columns (see k_rowmul_split).
+constexpr int kRowSplitMaxN = 64;
+cudaError_t launch_rowmul_split(const double* X, const double* M, const double* colsrc, const int* colexp, int64_t m,
+                                int n, bool add, double* out, int32_t* status, cudaStream_t st);
+// Step 3 for binary64 data, n <= kRowSplitMaxN; the block and tile geometry of
+// Step 1, Q over Y.
+cudaError_t launch_form_q_split(double* Y, int64_t m, int n, int64_t b, int B, int64_t bt, int kt, int64_t p,
+                                const double* T, const double* C, int64_t cblocks, int32_t* status, cudaStream_t st);
+// Partial Grams X^T Y into at most max_parts n x n partials (*parts written);
+// colexp (or NULL): n ints, zeroed by the caller, receiving the largest binary
+// exponents of X's columns.
+cudaError_t launch_gram_split(const double* X, const double* Y, int64_t m, int n, int max_parts, int* parts,
+                              double* part, int* colexp, cudaStream_t st);
+// The Gram entries of every tile's Householder vectors into the T slots'
+// strictly upper triangles.
+cudaError_t launch_gram_t_split(const double* Y, int64_t m, int n, int64_t b, int B, int64_t bt, int kt, int64_t p,
+                                double* T, cudaStream_t st);
 
 // Gram launch geometry shared by the planner and the launcher.
 struct GramGeom { int chunk, grid, nt, tile; };

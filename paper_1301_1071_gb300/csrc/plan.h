@@ -73,9 +73,13 @@ struct Plan {
   int prec = 0;          // the resolved tsqr_prec (TSQR_PREC_AUTO taken)
   bool tc3 = false;      // Step 3 on the tensor cores (3xTF32, binary32 data)
   bool oz3 = false;      // Step 3 on the tensor cores (Ozaki split, binary64 data, n <= 32)
-  // Step 1 without its Gram dot products and the T factors' Gram entries on
-  // the tensor cores (k_gram_oz): the Ozaki form with a one-row-group tile
-  bool gram_oz = false;
+  // binary64 arithmetic: Step 3 by digit products (k_form_q_split, n <=
+  // kRowSplitMaxN), and Step 1 without its Gram dot products, the T factors'
+  // Gram by digit products (k_gram_split; one-row-group tiles)
+  bool split3 = false, gram_split = false;
+  // the sign fix of the top R rides in the top level's T build (one launch
+  // less; the explicit Ozaki form keeps its own launch for it)
+  bool fuse_sign = false;
   // k_rowmul with two inputs (the adjoint): a register tile close to the
   // b_rm2 rows per block whose two inputs fit in shared memory together
   KernelCfg cfg_rm2;
@@ -103,7 +107,8 @@ constexpr int kMaxTiles = 64;       // binary64 data
 constexpr int kMaxTilesF32 = 128;   // binary32 data: its binary64 tree is costly, its rounding unit large
 constexpr int kMaxTilesDF64 = 8;
 constexpr int kDefaultSMs = 152;  // GB300
-constexpr int kMaxGramParts = 304;  // at most this many partial Grams (2 per SM of a GB300)
+constexpr int kMaxGramParts = 304;   // at most this many partial Grams (2 per SM of a GB300)
+constexpr int kMaxGramParts64 = 608;  // binary64 data (k_gram_split: up to 4 CTAs per SM)
 
 // TSQR_PREC_AUTO -> the concrete mode for this dtype and n (other modes
 // are returned unchanged): binary32 data at n >= kAutoTf32MinN takes the

@@ -8,8 +8,8 @@
 namespace tsqr {
 
 // ---------------------------------------------------------------------------
-__global__ void k_sign_fix(const double* __restrict__ Rraw, int n, double* __restrict__ Rout, int64_t ldr,
-                           double* __restrict__ Ctop, int32_t* status) {
+__device__ void cta_sign_fix(const double* __restrict__ Rraw, int n, double* __restrict__ Rout, int64_t ldr,
+                             double* __restrict__ Ctop, int32_t* status) {
   for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
     const int i = idx / n, k = idx % n;
     const double rik = Rraw[idx];
@@ -18,6 +18,11 @@ __global__ void k_sign_fix(const double* __restrict__ Rraw, int n, double* __res
     Rout[i * ldr + k] = (k >= i) ? d * rik : 0.0;
     Ctop[idx] = (i == k) ? d : 0.0;
   }
+}
+
+__global__ void k_sign_fix(const double* __restrict__ Rraw, int n, double* __restrict__ Rout, int64_t ldr,
+                           double* __restrict__ Ctop, int32_t* status) {
+  cta_sign_fix(Rraw, n, Rout, ldr, Ctop, status);
 }
 
 cudaError_t launch_sign_fix(const double* Rraw, int n, double* Rout, int64_t ldr, double* Ctop, int32_t* status,
@@ -594,8 +599,13 @@ __global__ void k_build_t(double* __restrict__ Tst, int64_t p, int n) {
 // to 0, T(i,c) = -tau_i sum_{k=i+1}^{c} G(i,k) T(k,c) (tau_i = 0 gives a zero
 // row, as the recursion does).  The sum runs over k ascending in two
 // interleaved chains.  G and T in shared memory, n x n each.
+// sf.Rout != NULL: one more CTA (the last) takes the sign fix of the top R.
 template <class F>
-__global__ void __launch_bounds__(128) k_build_t_cta(double* __restrict__ Tst, int n) {
+__global__ void __launch_bounds__(128) k_build_t_cta(double* __restrict__ Tst, int n, SignFix sf) {
+  if (sf.Rout && blockIdx.x + 1 == gridDim.x) {
+    cta_sign_fix(sf.Rraw, n, sf.Rout, sf.ldr, sf.Ctop, sf.status);
+    return;
+  }
   extern __shared__ __align__(16) unsigned char tsm_raw[];
   F* G = reinterpret_cast<F*>(tsm_raw);  // n x n: tau on the diagonal, G above it
   F* T = G + n * n;                       // n x n: column c is thread c's
@@ -626,14 +636,14 @@ __global__ void __launch_bounds__(128) k_build_t_cta(double* __restrict__ Tst, i
 }
 
 template <class F>
-static cudaError_t build_t_typed(double* Tst, int64_t p, int n, int sms, cudaStream_t st) {
+static cudaError_t build_t_typed(double* Tst, int64_t p, int n, int sms, const SignFix& sf, cudaStream_t st) {
   const size_t np = static_cast<size_t>(n) * (n + 1) / 2;
-  if (p < 2 * static_cast<int64_t>(sms)) {
+  if (p < 2 * static_cast<int64_t>(sms) || sf.Rout) {
     // few slots: latency decides, so one CTA per slot, a thread per column
     const size_t smem = 2 * static_cast<size_t>(n) * n * sizeof(F);
     cudaError_t e = cudaFuncSetAttribute(k_build_t_cta<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_build_t_cta<F><<<static_cast<unsigned>(p), 128, smem, st>>>(Tst, n);
+    k_build_t_cta<F><<<static_cast<unsigned>(p + (sf.Rout ? 1 : 0)), 128, smem, st>>>(Tst, n, sf);
     return cudaGetLastError();
   }
   // many slots: one warp per slot, as many warps (<= 16) as packed triangles fit in 220 KB
@@ -654,27 +664,36 @@ static cudaError_t build_t_typed(double* Tst, int64_t p, int n, int sms, cudaStr
   return cudaGetLastError();
 }
 
-cudaError_t launch_build_t(double* Tst, int64_t p, int n, bool binary32, cudaStream_t st) {
+cudaError_t launch_build_t(double* Tst, int64_t p, int n, bool binary32, cudaStream_t st, const SignFix& sf) {
   int dev = 0, sms = 152;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return binary32 ? build_t_typed<float>(Tst, p, n, sms, st) : build_t_typed<double>(Tst, p, n, sms, st);
+  return binary32 ? build_t_typed<float>(Tst, p, n, sms, sf, st) : build_t_typed<double>(Tst, p, n, sms, sf, st);
 }
 
 // G = sum over the nparts partials, in index order (one thread per entry).
+constexpr int kGrSlices = 16;
 __global__ void k_gram_reduce(const double* __restrict__ part, int nparts, int n, double* __restrict__ G,
                               int32_t* status) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= n * n) return;
+  // 32 entries per CTA, their partials in kGrSlices interleaved slices (one
+  // thread summed hundreds of partials in a chain of loads before), the slices
+  // in order: a fixed order for a given nparts
+  __shared__ double sl[kGrSlices][32];
+  const int el = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int e = blockIdx.x * 32 + el;
   double s = 0.0;
-  for (int p = 0; p < nparts; ++p) s += part[static_cast<int64_t>(p) * n * n + e];
+  if (e < n * n)
+    for (int p = w; p < nparts; p += kGrSlices) s += part[static_cast<int64_t>(p) * n * n + e];
+  sl[w][el] = s;
+  __syncthreads();
+  if (w != 0 || e >= n * n) return;
+  for (int k = 1; k < kGrSlices; ++k) s += sl[k][el];
   if (!isfinite(s)) set_status(status, TSQR_ERR_NONFINITE);
   G[e] = s;
 }
 
 cudaError_t launch_gram_reduce(const double* part, int nparts, int n, double* G, int32_t* status,
                                cudaStream_t st) {
-  const int threads = 256;
-  k_gram_reduce<<<(n * n + threads - 1) / threads, threads, 0, st>>>(part, nparts, n, G, status);
+  k_gram_reduce<<<(n * n + 31) / 32, 32 * kGrSlices, 0, st>>>(part, nparts, n, G, status);
   return cudaGetLastError();
 }
 
