@@ -38,6 +38,8 @@ cudaError_t launch_rowmul_f64(const KernelCfg&, const void*, const double*, cons
                               int, int64_t, int64_t, void*, int32_t*, cudaStream_t);
 cudaError_t launch_rowmul_f32(const KernelCfg&, const void*, const double*, const void*, const double*, int64_t,
                               int, int64_t, int64_t, void*, int32_t*, cudaStream_t);
+cudaError_t launch_gram_f64(const void*, const void*, int64_t, int, int, int, int, int, bool, double*, int32_t*,
+                            cudaStream_t);
 cudaError_t launch_gram_f32(const void*, const void*, int64_t, int, int, int, int, int, bool, double*, int32_t*,
                             cudaStream_t);
 
@@ -53,9 +55,12 @@ cudaError_t launch_gram(int esz, const void* X, const void* Y, int64_t m, int n,
   const GramGeom g = gram_geom(m, n, esz);
   int parts = g.grid;
   const cudaError_t e =
-      esz == 8 ? launch_gram_split(static_cast<const double*>(X), static_cast<const double*>(Y), m, n, g.grid, &parts,
-                                   part, colexp, st)
-               : launch_gram_f32(X, Y, m, n, g.chunk, g.grid, g.nt, g.tile, acc_storage, part, status, st);
+      esz == 8 && n >= kSplitMinN
+          ? launch_gram_split(static_cast<const double*>(X), static_cast<const double*>(Y), m, n, g.grid, &parts, part,
+                              colexp, st)
+      : esz == 8
+          ? launch_gram_f64(X, Y, m, n, g.chunk, g.grid, g.nt, g.tile, acc_storage, part, status, st)
+          : launch_gram_f32(X, Y, m, n, g.chunk, g.grid, g.nt, g.tile, acc_storage, part, status, st);
   if (e != cudaSuccess) return e;
   return launch_gram_reduce(part, parts, n, G, status, st);
 }
@@ -376,14 +381,14 @@ tsqr_status run_r_only(const Plan& P, int esz, const void* X, double* R, void* w
 
 // out = X M1 (+ Y M2): one input over the row blocks of the Step-1
 // configuration; two inputs with the tile sized for two staged inputs.
-// binary64 data with n <= kRowSplitMaxN: the digit products, one pass per input
+// binary64 data where rows_by_digits(n): the digit products, one pass per input
 // (xsrc / xexp: the scale of X's columns; Y's are orthonormal columns, their
 // own scale).  `out` may be one of the inputs: that one is then taken first,
 // while it is intact.
 tsqr_status rowmul(const Plan& P, const void* X, const double* M1, const void* Y, const double* M2, void* out,
                    int32_t* status, cudaStream_t st, const double* xsrc = nullptr, const int* xexp = nullptr) {
   const int ni = static_cast<int>(P.n);
-  if (P.esz == 8 && ni <= kRowSplitMaxN) {
+  if (P.esz == 8 && rows_by_digits(ni)) {
     const size_t bytes = static_cast<size_t>(P.m) * P.n * 8;
     auto clash = [&](const void* in) { return in && in != out && overlaps(in, bytes, out, bytes); };
     if (!clash(X) && !clash(Y) && !(X == out && Y == out)) {
@@ -586,8 +591,8 @@ tsqr_status tsqr_launch_count(int32_t op, int64_t m, int64_t n, int32_t dtype, c
     case TSQR_OP_SVD: *launches = 3 * L + 1 + s1 + g + w; break;  // + Jacobi SVD
     case TSQR_OP_CHOLQR: *launches = 4 * (1 + refine_steps) + refine_steps; break;  // gram, reduce, chol, rowmul (+ combine)
     case TSQR_OP_INDIRECT: *launches = (L + 3) * (1 + refine_steps) + refine_steps; break;
-    // gram, reduce, prep, rowmul (binary64, n <= kRowSplitMaxN: one pass per input)
-    case TSQR_OP_BACKWARD: *launches = P.esz == 8 && P.n <= kRowSplitMaxN ? 5 : 4; break;
+    // gram, reduce, prep, rowmul (rows_by_digits: one pass per input)
+    case TSQR_OP_BACKWARD: *launches = P.esz == 8 && rows_by_digits(P.n) ? 5 : 4; break;
     case TSQR_OP_R: *launches = L + 1; break;                 // L levels up (R only), sign fix
     case TSQR_OP_SVD_VALUES: *launches = L + 2; break;        // + Jacobi SVD
     default: return TSQR_ERR_ARG;
@@ -865,7 +870,7 @@ tsqr_status tsqr_backward(const void* Q, const double* R, const void* dQ, const 
   const int ni = static_cast<int>(n);
   TSQR_CUDA(cudaMemsetAsync(status, 0, sizeof(int32_t), st));
   // G = dQ^T Q; binary64: with the scale of dQ's columns, for the product below
-  int* qexp = esz == 8 && dQ ? reinterpret_cast<int*>(G + 3 * nn) : nullptr;
+  int* qexp = esz == 8 && dQ && rows_by_digits(n) ? reinterpret_cast<int*>(G + 3 * nn) : nullptr;
   if (qexp) TSQR_CUDA(cudaMemsetAsync(qexp, 0, n * sizeof(int), st));
   if (dQ) TSQR_CUDA(launch_gram(esz, dQ, Q, m, ni, part, G, status, st, esz == 4, qexp));
   TSQR_CUDA(launch_bwd_prep(R, dR, dQ ? G : nullptr, ni, M1, M2, status, st));

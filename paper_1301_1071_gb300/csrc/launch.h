@@ -74,7 +74,13 @@ cudaError_t launch_gram(int esz, const void* X, const void* Y, int64_t m, int n,
 
 // binary64 as exact digit products (split_kernels.cuh).  out (+)= X M, n <=
 // kRsMaxN: colsrc / colexp give the scale of X's columns (see k_rowmul_split).
+// kSplitMinN: below, the padding to 8 columns and 16 k steps costs more than
+// the binary64 unit (GB300, 20,000,000 x 4: Cholesky QR 2.6 ms by FMAs, 5.4 by
+// digits, direct 2.9 against 4.1; 10,000,000 x 6 direct 3.91 against 3.91; at
+// 10,000,000 x 8 5.1 against 4.6).
+constexpr int kSplitMinN = 7;
 constexpr int kRowSplitMaxN = 64;
+constexpr bool rows_by_digits(int64_t n) { return n >= kSplitMinN && n <= kRowSplitMaxN; }
 cudaError_t launch_rowmul_split(const double* X, const double* M, const double* colsrc, const int* colexp, int64_t m,
                                 int n, bool add, double* out, int32_t* status, cudaStream_t st);
 // Step 3 for binary64 data, n <= kRowSplitMaxN; the block and tile geometry of

@@ -139,10 +139,11 @@ GramGeom gram_geom(int64_t m, int n, int esz) {
   chunk = chunk > 1024 ? 1024 : chunk;
   chunk = chunk / 16 * 16;
   if (chunk < 16) chunk = 16;
-  if (esz == 8) chunk = n <= 64 ? 64 : 32;  // k_gram_split
+  const bool digits = esz == 8 && n >= kSplitMinN;
+  if (digits) chunk = n <= 64 ? 64 : 32;  // k_gram_split
   g.chunk = (int)chunk;
   const int64_t nchunks = (m + chunk - 1) / chunk;
-  const int most = esz == 8 ? kMaxGramParts64 : kMaxGramParts;
+  const int most = digits ? kMaxGramParts64 : kMaxGramParts;
   g.grid = (int)(nchunks < most ? nchunks : most);
   const int n4 = (n + 3) / 4, n5 = (n + 4) / 5;
   g.tile = (n5 * n5 * 25 < n4 * n4 * 16) ? 5 : 4;  // fewer padded products
@@ -229,11 +230,11 @@ int make_plan(int64_t m, int64_t n, int esz, int64_t block_rows, int fanout, Pla
 
   P.prec = prec;
   P.tc3 = prec == TSQR_PREC_TF32X3 && n <= kTcwMaxN;
-  P.oz3 = prec == TSQR_PREC_OZAKI && n <= kOzMaxN;
+  P.oz3 = prec == TSQR_PREC_OZAKI && n >= kSplitMinN && n <= kOzMaxN;
   // binary64 arithmetic: Step 3 and (Step 1's one-row-group tiles) the T
   // factors' Gram as exact digit products
-  P.split3 = kind0 == kKindF64 && n <= kRowSplitMaxN;
-  P.gram_split = kind0 == kKindF64 && P.cfg0.NRG == 1;
+  P.split3 = kind0 == kKindF64 && rows_by_digits(n);
+  P.gram_split = kind0 == kKindF64 && n >= kSplitMinN && P.cfg0.NRG == 1;
   P.fuse_sign = P.gram_split && !P.oz3;
   {
     const int kind_rm = esz == 4 ? kKindF32 : kKindF64;
