@@ -121,7 +121,8 @@ def load_peaks():
 # traffic bench.py reports from a committed ncu capture.
 KERNEL_SOURCES = ["qr_kernels.cuh", "device.cuh", "df64.cuh", "layout.cuh", "kern_inst.cuh", "kern_f64.cu",
                   "kern_df64.cu", "kern_f32.cu", "kern_r_f64.cu", "tiles_f64.h", "tiles_f32.h", "plan.cu", "plan.h",
-                  "oz_kernels.cuh", "kern_oz.cu", "tcgen05.cuh", "chunks.cuh"]
+                  "split.cuh", "split_kernels.cuh", "kern_split.cu", "panel64.cuh", "kern_panel64.cu", "tcgen05.cuh",
+                  "chunks.cuh"]
 
 
 def kernel_source_hash() -> str:
@@ -468,7 +469,7 @@ def main():
         "vs_baseline": None,
         "dtype": ("df64 (binary64 data, pairs of binary32 in Steps 1 and 3, binary64 tree)" if resolved == "df64"
                   else "f64 (binary64 Householder and tree; the Step-3 product and the T factors' Gram as "
-                       "error-free Ozaki splits on tcgen05: 56/64-bit fixed point, exact binary32 accumulation, "
+                       "error-free Ozaki splits on the tensor cores: 62-bit fixed point, exact binary32 accumulation, "
                        "one rounding to binary64)" if resolved == "ozaki"
                   else "f32 (Step 3 product as 3xTF32 on the tensor cores)" if resolved == "tf32x3"
                   else ("f64" if elem == 8 else "f32")),

@@ -79,8 +79,13 @@ typedef enum tsqr_dtype { TSQR_F64 = 0, TSQR_F32 = 1 } tsqr_dtype;
 /* Arithmetic of the tall passes (Step 1 and Step 3).  Only tsqr_direct and
  * tsqr_svd honour it; the Step-2 tree, the SVD of R and all n x n work are
  * binary64 in every mode.
- * NATIVE: the data's type (binary64 for TSQR_F64, binary32 with binary32
- *         accumulation for TSQR_F32).
+ * NATIVE: the data's type (binary32 with binary32 accumulation for TSQR_F32).
+ *         TSQR_F64: binary64 accuracy; from n = 7 on the matrix products of
+ *         the tall passes (the trailing updates of Step 1 for most n, T's Gram,
+ *         Step 3 for n <= 64) are exact sums of 8-bit digit products on the
+ *         tensor cores (Ozaki, Ogita, Oishi, Rump 2012: 54- to 62-bit fixed
+ *         point, binary16 operands, exact binary32 sums, one rounding to
+ *         binary64), the factorisation of a panel of columns in binary64.
  * DF64:   TSQR_F64 data only.  Binary64 storage, double-float arithmetic
  *         (pairs of binary32, ~48-bit significand) in Step 1 and Step 3, each
  *         row block scaled by a power of two (exact).  Targets ||Q^TQ - I||
@@ -92,16 +97,9 @@ typedef enum tsqr_dtype { TSQR_F64 = 0, TSQR_F32 = 1 } tsqr_dtype;
  * AUTO:   the library's choice for the data: TSQR_F32 data takes TF32X3 at
  *         n >= 20 (where it is the faster Step 3) and NATIVE below;
  *         TSQR_F64 data takes OZAKI at n <= 32 and NATIVE above.
- * OZAKI:  TSQR_F64 data only.  Step 1's Householder factorisation and the
- *         tree in binary64; for n <= 32 the two products of the method run on
- *         the tensor cores as error-free split products (Ozaki, Ogita, Oishi,
- *         Rump 2012): the Step-3 product Y_i W_i (each row of Y and column of
- *         W cut into 7 digits of 8 bits, 56 bits, against its largest
- *         exponent) and the Gram entries V^T V of the compact-WY T factors
- *         (8 digits, 64 bits; Step 1 then leaves them out of its column
- *         loop).  The digit products accumulate exactly in binary32
- *         (binary16 operands), are recombined in 64-bit integers and rounded
- *         once to binary64.  Above n = 32, NATIVE. */
+ * OZAKI:  TSQR_F64 data only.  Names that arithmetic for n <= 32 (the same
+ *         kernels and results as NATIVE; the sign fix of R is a launch of its
+ *         own).  Above n = 32, NATIVE. */
 typedef enum tsqr_prec {
   TSQR_PREC_NATIVE = 0,
   TSQR_PREC_DF64 = 1,
@@ -356,7 +354,9 @@ tsqr_status tsqr_launch_count(int32_t op, int64_t m, int64_t n, int32_t dtype, c
  *   tree_levels     Step-2 tree levels (0: a single block, no tree)
  *   tree_fanout     R factors merged per tree node
  *   prec            the tsqr_prec the call computes in (TSQR_PREC_AUTO resolved)
- *   step3_tensor    1 when Step 3 runs on the tensor cores
+ *   step3_tensor    1 when `prec` names a tensor-core form of Step 3 (TF32X3, or
+ *                   OZAKI in its range); NATIVE reports 0 also where its
+ *                   binary64 products are digit products
  */
 typedef struct tsqr_plan_info {
   int64_t block_rows;

@@ -19,21 +19,19 @@ cudaError_t launch_local_qr_f64(const KernelCfg&, const void*, int64_t, int, int
                                 double*, int32_t*, cudaStream_t);
 cudaError_t launch_local_qr_f32(const KernelCfg&, const void*, int64_t, int, int64_t, int64_t, int, int64_t, void*, double*,
                                 double*, int32_t*, cudaStream_t);
-cudaError_t launch_form_q_f64(const KernelCfg&, const void*, int64_t, int, int64_t, int64_t, int, int64_t, const double*,
+cudaError_t launch_form_q_f64(const KernelCfg&, const void*, int64_t, int, int64_t, int, int64_t, int, int64_t, const double*,
                               const double*, int64_t, void*, int32_t*, cudaStream_t);
-cudaError_t launch_form_q_f32(const KernelCfg&, const void*, int64_t, int, int64_t, int64_t, int, int64_t, const double*,
+cudaError_t launch_form_q_f32(const KernelCfg&, const void*, int64_t, int, int64_t, int, int64_t, int, int64_t, const double*,
                               const double*, int64_t, void*, int32_t*, cudaStream_t);
 
 cudaError_t launch_local_qr_df64(const KernelCfg&, const void*, int64_t, int, int64_t, int64_t, int, int64_t, void*, double*,
                                  double*, int32_t*, cudaStream_t);
-cudaError_t launch_form_q_df64(const KernelCfg&, const void*, int64_t, int, int64_t, int64_t, int, int64_t, const double*,
+cudaError_t launch_form_q_df64(const KernelCfg&, const void*, int64_t, int, int64_t, int, int64_t, int, int64_t, const double*,
                                const double*, int64_t, void*, int32_t*, cudaStream_t);
 cudaError_t launch_local_r_f64(const KernelCfg&, const void*, int64_t, int, int64_t, int64_t, int, int64_t, double*,
                                int32_t*, cudaStream_t);
 cudaError_t launch_local_r_f32(const KernelCfg&, const void*, int64_t, int, int64_t, int64_t, int, int64_t, double*,
                                int32_t*, cudaStream_t);
-cudaError_t launch_local_qr_nogram_f64(const KernelCfg&, const void*, int64_t, int, int64_t, int64_t, int, int64_t,
-                                       void*, double*, double*, int32_t*, cudaStream_t);
 cudaError_t launch_rowmul_f64(const KernelCfg&, const void*, const double*, const void*, const double*, int64_t,
                               int, int64_t, int64_t, void*, int32_t*, cudaStream_t);
 cudaError_t launch_rowmul_f32(const KernelCfg&, const void*, const double*, const void*, const double*, int64_t,
@@ -42,6 +40,9 @@ cudaError_t launch_gram_f64(const void*, const void*, int64_t, int, int, int, in
                             cudaStream_t);
 cudaError_t launch_gram_f32(const void*, const void*, int64_t, int, int, int, int, int, bool, double*, int32_t*,
                             cudaStream_t);
+
+cudaError_t launch_local_qr_nogram_f64(const KernelCfg&, const void*, int64_t, int, int64_t, int64_t, int, int64_t, void*,
+                                       double*, double*, int32_t*, cudaStream_t);
 
 cudaError_t launch_rowmul(const KernelCfg& k, const void* X, const double* M1, const void* Y,
                           const double* M2, int64_t m, int n, int64_t b, int64_t p, void* out, int32_t* status,
@@ -90,8 +91,9 @@ cudaError_t launch_local_qr_step1(const Plan& P, const void* A, int64_t m, int64
                                   double* Rst, double* Tst, int32_t* status, cudaStream_t st) {
   const Level& l0 = P.levels[0];
   const int n = static_cast<int>(P.n);
-  if (!P.gram_split) return launch_local_qr(P.cfg0, A, m, n, b, l0.bt, l0.kt, p, Y, Rst, Tst, status, st);
-  return launch_local_qr_nogram_f64(P.cfg0, A, m, n, b, l0.bt, l0.kt, p, Y, Rst, Tst, status, st);
+  return P.panel        ? launch_panel_qr_f64(P.pq, A, m, n, b, l0.kt, p, Y, Rst, Tst, status, st)
+         : P.gram_split ? launch_local_qr_nogram_f64(P.cfg0, A, m, n, b, l0.bt, l0.kt, p, Y, Rst, Tst, status, st)
+                        : launch_local_qr(P.cfg0, A, m, n, b, l0.bt, l0.kt, p, Y, Rst, Tst, status, st);
 }
 
 cudaError_t launch_step1(const Plan& P, const void* A, int64_t m, int64_t b, int64_t p, void* Y, double* Rst,
@@ -100,16 +102,16 @@ cudaError_t launch_step1(const Plan& P, const void* A, int64_t m, int64_t b, int
   const int n = static_cast<int>(P.n);
   cudaError_t e = launch_local_qr_step1(P, A, m, b, p, Y, Rst, Tst, status, st);
   if (e != cudaSuccess || !P.gram_split) return e;
-  return launch_gram_t_split(static_cast<const double*>(Y), m, n, b, P.cfg0.B, l0.bt, l0.kt, p, Tst, st);
+  return launch_gram_t_split(static_cast<const double*>(Y), m, n, b, P.B0, l0.bt, l0.kt, p, Tst, st);
 }
 
-cudaError_t launch_form_q(const KernelCfg& k, const void* Y, int64_t m, int n, int64_t b, int64_t bt, int kt,
+cudaError_t launch_form_q(const KernelCfg& k, const void* Y, int64_t m, int n, int64_t b, int B, int64_t bt, int kt,
                           int64_t p, const double* T, const double* C, int64_t cblocks, void* Q, int32_t* status,
                           cudaStream_t st) {
   switch (k.kind) {
-    case kKindF64: return launch_form_q_f64(k, Y, m, n, b, bt, kt, p, T, C, cblocks, Q, status, st);
-    case kKindF32: return launch_form_q_f32(k, Y, m, n, b, bt, kt, p, T, C, cblocks, Q, status, st);
-    case kKindDF64: return launch_form_q_df64(k, Y, m, n, b, bt, kt, p, T, C, cblocks, Q, status, st);
+    case kKindF64: return launch_form_q_f64(k, Y, m, n, b, B, bt, kt, p, T, C, cblocks, Q, status, st);
+    case kKindF32: return launch_form_q_f32(k, Y, m, n, b, B, bt, kt, p, T, C, cblocks, Q, status, st);
+    case kKindDF64: return launch_form_q_df64(k, Y, m, n, b, B, bt, kt, p, T, C, cblocks, Q, status, st);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -315,7 +317,7 @@ tsqr_status run_direct(const Plan& P, const void* A, void* Q, double* R, int64_t
   if (mark(o, 1, st) != TSQR_OK) return TSQR_ERR_CUDA;
   // the T factors' Gram entries on the tensor cores (Ozaki form); like the T
   // build below, it is part of the Step-2 interval of the stage events
-  if (P.gram_split && launch_gram_t_split(static_cast<const double*>(Q), P.m, n, l0.b, P.cfg0.B, l0.bt, l0.kt, l0.p,
+  if (P.gram_split && launch_gram_t_split(static_cast<const double*>(Q), P.m, n, l0.b, P.B0, l0.bt, l0.kt, l0.p,
                                           T(0), st) != cudaSuccess)
     return TSQR_ERR_CUDA;
   // The row blocks' T factors are read only by Step 3 and the tree reads only
@@ -343,11 +345,11 @@ tsqr_status run_direct(const Plan& P, const void* A, void* Q, double* R, int64_t
   double* C0 = (L == 1) ? ctop : S(0);
   const int64_t cb0 = (L == 1) ? 1 : l0.p;
   const cudaError_t e3 =
-      P.split3 ? launch_form_q_split(static_cast<double*>(Q), P.m, n, l0.b, P.cfg0.B, l0.bt, l0.kt, l0.p, T(0), C0, cb0,
+      P.split3 ? launch_form_q_split(static_cast<double*>(Q), P.m, n, l0.b, P.B0, l0.bt, l0.kt, l0.p, T(0), C0, cb0,
                                      status, st)
-      : P.tc3 ? launch_form_q_tc(static_cast<float*>(Q), P.m, n, l0.b, P.cfg0.B, l0.bt, l0.kt, l0.p, T(0), C0, cb0,
+      : P.tc3 ? launch_form_q_tc(static_cast<float*>(Q), P.m, n, l0.b, P.B0, l0.bt, l0.kt, l0.p, T(0), C0, cb0,
                                  status, st)
-              : launch_form_q(P.cfg0, Q, P.m, n, l0.b, l0.bt, l0.kt, l0.p, T(0), C0, cb0, Q, status, st);
+              : launch_form_q(P.cfg0, Q, P.m, n, l0.b, P.B0, l0.bt, l0.kt, l0.p, T(0), C0, cb0, Q, status, st);
   if (e3 != cudaSuccess) return TSQR_ERR_CUDA;
   return mark(o, 3, st);
 }
@@ -363,7 +365,8 @@ tsqr_status run_r_only(const Plan& P, int esz, const void* X, double* R, void* w
   double* ctop = reinterpret_cast<double*>(at(work, P.off_ctop));
   const Level& l0 = P.levels[0];
   const cudaError_t e0 =
-      launch_local_qr(P.cfg0, X, P.m, n, l0.b, l0.bt, l0.kt, l0.p, nullptr, S(0), nullptr, status, st);
+      P.panel ? launch_panel_qr_f64(P.pq, X, P.m, n, l0.b, l0.kt, l0.p, nullptr, S(0), nullptr, status, st)
+              : launch_local_qr(P.cfg0, X, P.m, n, l0.b, l0.bt, l0.kt, l0.p, nullptr, S(0), nullptr, status, st);
   if (e0 != cudaSuccess) return TSQR_ERR_CUDA;
   for (size_t l = 1; l < L; ++l) {
     const Level& lv = P.levels[l];
@@ -512,11 +515,11 @@ tsqr_status run_direct_host(const Plan& P, int chunks, const char* A, char* Qh, 
     double* Cc = (L == 1) ? C0 : C0 + b0 * nn;
     const int64_t cb = (L == 1) ? 1 : pcnt;
     char* Y = dbuf + r0 * row_bytes;
-    TSQR_CUDA(P.split3 ? launch_form_q_split(reinterpret_cast<double*>(Y), rows, n, l0.b, P.cfg0.B, l0.bt, l0.kt,
+    TSQR_CUDA(P.split3 ? launch_form_q_split(reinterpret_cast<double*>(Y), rows, n, l0.b, P.B0, l0.bt, l0.kt,
                                              pcnt, T0 + b0 * l0.kt * nn, Cc, cb, status, st)
-              : P.tc3 ? launch_form_q_tc(reinterpret_cast<float*>(Y), rows, n, l0.b, P.cfg0.B, l0.bt, l0.kt, pcnt,
+              : P.tc3 ? launch_form_q_tc(reinterpret_cast<float*>(Y), rows, n, l0.b, P.B0, l0.bt, l0.kt, pcnt,
                                          T0 + b0 * l0.kt * nn, Cc, cb, status, st)
-                      : launch_form_q(P.cfg0, Y, rows, n, l0.b, l0.bt, l0.kt, pcnt, T0 + b0 * l0.kt * nn, Cc, cb, Y,
+                      : launch_form_q(P.cfg0, Y, rows, n, l0.b, P.B0, l0.bt, l0.kt, pcnt, T0 + b0 * l0.kt * nn, Cc, cb, Y,
                                       status, st));
     TSQR_CUDA(cudaEventRecord(ev_q[c], st));
     TSQR_CUDA(cudaStreamWaitEvent(cst, ev_q[c], 0));

@@ -15,8 +15,12 @@ namespace tsqr {
 // (T slots per block).
 cudaError_t launch_local_qr(const KernelCfg& k, const void* A, int64_t m, int n, int64_t b, int64_t bt, int kt,
                             int64_t p, void* Y, double* Rst, double* Tst, int32_t* status, cudaStream_t st);
-// Step 3 / tree down-pass: p CTAs.
-cudaError_t launch_form_q(const KernelCfg& k, const void* Y, int64_t m, int n, int64_t b, int64_t bt, int kt,
+// Step 1 of binary64 data by panels (tiles of kPdRows rows, kt T slots per block):
+// Y, R and tau, or (Y == NULL) R only.
+cudaError_t launch_panel_qr_f64(const PanelCfg& k, const void* A, int64_t m, int n, int64_t b, int kt, int64_t p,
+                                void* Y, double* Rst, double* Tst, int32_t* status, cudaStream_t st);
+// Step 3: p CTAs (B, bt: the tile geometry of Step 1).
+cudaError_t launch_form_q(const KernelCfg& k, const void* Y, int64_t m, int n, int64_t b, int B, int64_t bt, int kt,
                           int64_t p, const double* T, const double* C, int64_t cblocks, void* Q,
                           int32_t* status, cudaStream_t st);
 
@@ -47,19 +51,6 @@ cudaError_t launch_tree_down(double* Y, int64_t rows, int n, int f, int64_t p, c
 // n <= 64 the T slots and C are overwritten (with W and X_0).
 cudaError_t launch_form_q_tc(float* Y, int64_t m, int n, int64_t b, int B, int64_t bt, int kt, int64_t p,
                              double* T, double* C, int64_t cblocks, int32_t* status, cudaStream_t st);
-
-// Step 3 for binary64 data with the product Y W on the tensor cores by
-// Ozaki splitting (binary16 digits, exact binary32 accumulation), n <= 32;
-// the block and tile geometry of Step 1.
-cudaError_t launch_form_q_oz(double* Y, int64_t m, int n, int64_t b, int B, int64_t bt, int kt, int64_t p,
-                             const double* T, const double* C, int64_t cblocks, int32_t* status, cudaStream_t st);
-
-// The Gram entries v_i^T v_c (i < c) of every tile's Householder vectors
-// into the T slots' strictly upper triangles (binary64 data, n <= 32), on the
-// tensor cores by Ozaki splitting; Step 1 ran without its Gram dot products
-// (launch_local_qr_nogram_f64, which writes Y, R and tau).
-cudaError_t launch_gram_oz(const double* Y, int64_t m, int n, int64_t b, int B, int64_t bt, int kt, int64_t p,
-                           double* T, int32_t* status, cudaStream_t st);
 
 // out_r = X_r M1 + Y_r M2 over p blocks of b rows (X or Y may be NULL).
 cudaError_t launch_rowmul(const KernelCfg& k, const void* X, const double* M1, const void* Y,

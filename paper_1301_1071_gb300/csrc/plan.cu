@@ -8,7 +8,7 @@
 #include "../../include/tsqr.h"
 #include "launch.h"
 #include "layout.cuh"
-#include "oz_kernels.cuh"
+#include "panel64.cuh"
 #include "tc_kernels.cuh"
 
 namespace tsqr {
@@ -133,6 +133,23 @@ bool choose_cfg(int kind, int n, KernelCfg* out, int64_t want_b, int policy, int
   return true;
 }
 
+// 16 warps of 128 registers an SM: as many CTAs as those and the shared memory
+// allow (one ring slot is enough to run: it is held from publication to the
+// last reader only), then ring slots up to one and a half a published panel.
+PanelCfg choose_panel(int n) {
+  PanelCfg c;
+  c.NW = (n + kPdCols - 1) / kPdCols;
+  const int entries = c.NW - 1;  // published panels per tile
+  for (c.ctas = kPdMaxThreads / 32 / c.NW; c.ctas >= 1; --c.ctas) {
+    const size_t lim = c.ctas == 1 ? kSmemMax : kSmemPerSM / c.ctas - 1024;
+    for (c.NS = entries + entries / 2 + 1; c.NS >= 1; --c.NS) {
+      c.smem = Panel64Smem(c.NW, c.NS).total;
+      if (c.smem <= lim) return c;
+    }
+  }
+  return c;  // not reached: one CTA holds at least one slot for every n
+}
+
 GramGeom gram_geom(int64_t m, int n, int esz) {
   GramGeom g;
   int64_t chunk = (int64_t)(kSmemMax - 64) / (2 * (int64_t)n * esz);
@@ -166,6 +183,43 @@ int resolve_prec(int prec, int esz, int64_t n) {
   return n <= kOzMaxN ? TSQR_PREC_OZAKI : TSQR_PREC_NATIVE;
 }
 
+// Default block height of the panel form: k tiles a block for the least
+// waves(k) k + 3.2 levels(k).  A tile costs a resident CTA about 3 n us through
+// Steps 1 and 3 (n = 8 .. 64: 32, 63, 156, 200 us at n = 8, 25, 50, 64), a tree
+// level about 9.5 n us (n = 25, 50, 64: 230, 465, 760).  30,000 x 50: one tile a
+// block, 4 levels 2.27 ms, two tiles, 3 levels 1.88; 100,000 x 25: 3 levels
+// 1.19 ms, 2 levels 0.89.  At most kMaxTiles tiles (the rounding of a block's
+// chain grows with them).
+static int64_t panel_block_rows(int64_t m, int64_t f, int64_t slots, int64_t al) {
+  auto levels = [&](int64_t p) {  // in rounds of kDefaultSMs nodes
+    int64_t l = 0;
+    for (; p > 1;) {
+      p = (p + f - 1) / f;
+      l += (p + kDefaultSMs - 1) / kDefaultSMs;
+    }
+    return l;
+  };
+  double best = 0;
+  int64_t rows = kPdRows;
+  for (int64_t k = 1; k <= kMaxTiles; ++k) {
+    const int64_t p = (m + k * kPdRows - 1) / (k * kPdRows);
+    const int64_t waves = (p + slots - 1) / slots;
+    const double cost = (double)waves * (double)k + 3.2 * (double)levels(p);
+    if (k == 1 || cost < best) {
+      best = cost;
+      rows = k * kPdRows;
+      // blocks of even height over whole waves, where that adds no level
+      const int64_t q = waves * slots;
+      if (waves > 1 && levels(q) == levels(p)) {
+        const int64_t b = (m + q - 1) / q;
+        rows = (b + al - 1) / al * al;
+      }
+    }
+    if (p == 1) break;
+  }
+  return rows;
+}
+
 int make_plan(int64_t m, int64_t n, int esz, int64_t block_rows, int fanout, Plan* plan, int prec, int sms) {
   if (n < 1 || n > TSQR_NMAX || m < n) return TSQR_ERR_SHAPE;
   // every m x n matrix of the call, at 8 bytes an entry, must have a byte
@@ -188,25 +242,47 @@ int make_plan(int64_t m, int64_t n, int esz, int64_t block_rows, int fanout, Pla
     return TSQR_ERR_SHAPE;
   if (block_rows > 0 && block_rows <= P.cfg0.B && !choose_cfg(kind0, (int)n, &P.cfg0, block_rows, kPolicyStep1))
     return TSQR_ERR_SHAPE;
-  const int64_t B0 = P.cfg0.B;
+  // binary64 Step 1: panels of 8 columns, or the column-by-column register
+  // tile (5 columns a warp) where that pads clearly less.  Step 1 of 3,000,000
+  // rows, tile -> panels: n = 8 0.81 -> 0.72 ms, 10 0.87 -> 1.54, 12 1.75 -> 1.67,
+  // 16 3.03 -> 1.88, 17 2.87 -> 3.40, 20 3.19 -> 3.74, 24 5.43 -> 3.85, 25 5.41 ->
+  // 5.28 (with more, shorter tiles for the T factors and Step 3 to take), 28
+  // 7.26 -> 5.88, 32 10.96 -> 5.70, 48 30.9 -> 11.5
+  P.panel = kind0 == kKindF64 && n >= kSplitMinN &&
+            !(n <= 25 && (n + 4) / 5 * 5 + 3 < (n + kPdCols - 1) / kPdCols * kPdCols);
+  if (P.panel) P.pq = choose_panel((int)n);
+  P.B0 = P.panel ? kPdRows : P.cfg0.B;
+  P.ctas0 = P.panel ? P.pq.ctas : P.cfg0.ctas;
+  const int64_t B0 = P.B0;
   // rows per tile after the first: the register tile less the carried R,
   // rounded down so that every tile starts on a 16-byte boundary when the
   // block does (bulk copies)
   int64_t al = 1;
   while ((al * n * esz) % 16 != 0) ++al;
-  const int64_t bt = (B0 - n) / al * al;
+  // (the panel form keeps R out of the tile)
+  const int64_t bt = (P.panel ? B0 : B0 - n) / al * al;
   if (bt < 1) return TSQR_ERR_SHAPE;
+  // tree node = f stacked R factors, f >= 2: up to the binary64 row-block
+  // tile's rows (fmax), or any f whose node fits one CTA's shared memory or
+  // a cluster of f CTAs.  Default: fmax while a node of 4 triangles fits one
+  // CTA, else (n > 84, where one CTA holds at most 3) nodes of kTreeClMaxF
+  // triangles on clusters: 20,000,000 x 100 has 4 tree levels instead of 10
+  const int64_t fmax = P.cfg64.B / n;
+  const int ni = static_cast<int>(n);
+  const int64_t f = fanout > 0 ? fanout : (fmax >= 4 && tree_up_fits(ni, 4) ? fmax : kTreeClMaxF);
   int64_t b0 = block_rows;
-  if (b0 <= 0) {
+  if (b0 <= 0 && P.panel) {
+    b0 = panel_block_rows(m, f, (int64_t)(sms < 1 ? kDefaultSMs : sms) * P.ctas0, al);
+  } else if (b0 <= 0) {
     if (sms < 1) sms = kDefaultSMs;
     const int64_t kmax = kind0 == kKindDF64 ? kMaxTilesDF64 : (kind0 == kKindF32 ? kMaxTilesF32 : kMaxTiles);
     const int64_t bmax = B0 + (kmax - 1) * bt;
-    if (m <= (int64_t)kMinWaves * sms * P.cfg0.ctas * B0) {
+    if (m <= (int64_t)kMinWaves * sms * P.ctas0 * B0) {
       b0 = B0;
     } else {
-      const int64_t slots = (int64_t)sms * P.cfg0.ctas;  // CTAs resident at once
+      const int64_t slots = (int64_t)sms * P.ctas0;  // CTAs resident at once
       int64_t waves = (m + slots * bmax - 1) / (slots * bmax);
-      const int64_t wmin = (kMinWaves + P.cfg0.ctas - 1) / P.cfg0.ctas;  // kMinWaves blocks per SM
+      const int64_t wmin = (kMinWaves + P.ctas0 - 1) / P.ctas0;  // kMinWaves blocks per SM
       if (waves < wmin) waves = wmin;
       const int64_t p = waves * slots;
       b0 = (m + p - 1) / p;
@@ -216,15 +292,8 @@ int make_plan(int64_t m, int64_t n, int esz, int64_t block_rows, int fanout, Pla
   if (b0 < n) return TSQR_ERR_SHAPE;
   if (b0 > m) b0 = m;  // one block
   const int64_t kt0 = b0 <= B0 ? 1 : 1 + (b0 - B0 + bt - 1) / bt;
-  if (kt0 > (1 << 20)) return TSQR_ERR_SHAPE;
-  // tree node = f stacked R factors, f >= 2: up to the binary64 row-block
-  // tile's rows (fmax), or any f whose node fits one CTA's shared memory or
-  // a cluster of f CTAs.  Default: fmax while a node of 4 triangles fits one
-  // CTA, else (n > 84, where one CTA holds at most 3) nodes of kTreeClMaxF
-  // triangles on clusters: 20,000,000 x 100 has 4 tree levels instead of 10
-  const int64_t fmax = P.cfg64.B / n;
-  const int ni = static_cast<int>(n);
-  const int64_t f = fanout > 0 ? fanout : (fmax >= 4 && tree_up_fits(ni, 4) ? fmax : kTreeClMaxF);
+  // tiles per block: heights up to 2^31 - 1 rows in either form
+  if (kt0 > (P.panel ? 1 << 24 : 1 << 20)) return TSQR_ERR_SHAPE;
   if (f < 2 || (f > fmax && !tree_up_fits(ni, static_cast<int>(f)) && !tree_up_cl_fits(ni, static_cast<int>(f))))
     return TSQR_ERR_SHAPE;
 
@@ -234,7 +303,7 @@ int make_plan(int64_t m, int64_t n, int esz, int64_t block_rows, int fanout, Pla
   // binary64 arithmetic: Step 3 and (Step 1's one-row-group tiles) the T
   // factors' Gram as exact digit products
   P.split3 = kind0 == kKindF64 && rows_by_digits(n);
-  P.gram_split = kind0 == kKindF64 && n >= kSplitMinN && P.cfg0.NRG == 1;
+  P.gram_split = kind0 == kKindF64 && n >= kSplitMinN && (P.panel || P.cfg0.NRG == 1);
   P.fuse_sign = P.gram_split && !P.oz3;
   {
     const int kind_rm = esz == 4 ? kKindF32 : kKindF64;
@@ -312,7 +381,7 @@ int make_host_plan(int64_t m, int64_t n, int esz, int64_t block_rows, int fanout
   int rc = make_plan(m, n, esz, block_rows, fanout, &P0, prec, sms);
   if (rc != TSQR_OK) return rc;
   if (sms < 1) sms = kDefaultSMs;
-  const int64_t slots = (int64_t)sms * P0.cfg0.ctas;
+  const int64_t slots = (int64_t)sms * P0.ctas0;
   if (block_rows <= 0) {
     int64_t c = (m * n * esz) / kHostChunkBytes;
     c = c < 1 ? 1 : (c > kMaxHostChunks ? kMaxHostChunks : c);
@@ -325,7 +394,7 @@ int make_host_plan(int64_t m, int64_t n, int esz, int64_t block_rows, int fanout
       while ((al * n * esz) % 16 != 0) ++al;
       int64_t b = (m + p - 1) / p;
       b = (b + al - 1) / al * al;
-      if (b >= n && b >= P0.cfg0.B) {
+      if (b >= n && b >= P0.B0) {
         Plan P1;
         if (make_plan(m, n, esz, b, fanout, &P1, prec, sms) == TSQR_OK) P0 = P1;
       }

@@ -52,6 +52,14 @@ enum { kPolicyStep1 = 0, kPolicyLargest = 1, kPolicyInFlight = 2 };
 // smallest per-CTA capacity that holds want_b rows; else `policy`).
 bool choose_cfg(int kind, int n, KernelCfg* out, int64_t want_b = 0, int policy = kPolicyStep1, int min_b = 0);
 
+// Launch shape of k_panel_qr_f64 (Step 1 of binary64 data): panel warps, ring
+// slots, CTAs per SM, shared memory.
+struct PanelCfg {
+  int NW = 0, NS = 0, ctas = 1;
+  size_t smem = 0;
+};
+PanelCfg choose_panel(int n);
+
 struct Level {
   int64_t rows = 0;  // rows of this level's input matrix
   int64_t b = 0;     // rows per block
@@ -72,7 +80,12 @@ struct Plan {
   KernelCfg cfg64;       // tree kernel config (binary64)
   int prec = 0;          // the resolved tsqr_prec (TSQR_PREC_AUTO taken)
   bool tc3 = false;      // Step 3 on the tensor cores (3xTF32, binary32 data)
-  bool oz3 = false;      // Step 3 on the tensor cores (Ozaki split, binary64 data, n <= 32)
+  bool oz3 = false;      // TSQR_PREC_OZAKI in its range (binary64 data, kSplitMinN <= n <= kOzMaxN)
+  // Step 1 by panels (k_panel_qr_f64), and Step 1's geometry: rows per
+  // register tile and CTAs per SM
+  bool panel = false;
+  PanelCfg pq;
+  int B0 = 0, ctas0 = 1;
   // binary64 arithmetic: Step 3 by digit products (k_form_q_split, n <=
   // kRowSplitMaxN), and Step 1 without its Gram dot products, the T factors'
   // Gram by digit products (k_gram_split; one-row-group tiles)
@@ -116,6 +129,8 @@ constexpr int kMaxGramParts64 = 608;  // binary64 data (k_gram_split: up to 4 CT
 // n = 16 on; below, the chunk stream's per-chunk cost dominates), binary64
 // data at n <= 32 the Ozaki form, everything else the data's own arithmetic.
 constexpr int kAutoTf32MinN = 20;
+// the Ozaki mode's range (above: native)
+constexpr int kOzMaxN = 32;
 int resolve_prec(int prec, int esz, int64_t n);
 
 // Workspace bytes of `op` (tsqr_op) under a built plan.

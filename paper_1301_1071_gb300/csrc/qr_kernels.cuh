@@ -130,6 +130,59 @@ __device__ __forceinline__ Reflector<T> make_reflector(T Sj, T alpha) {
   }
   return f;
 }
+// binary64 <-> binary32 by integer operations (normal numbers in binary32's
+// range; towards zero): a conversion costs a slot of the binary64 unit.
+__device__ __forceinline__ float float_of(double x) {
+  const uint32_t hi = static_cast<uint32_t>(__double2hiint(x)), lo = static_cast<uint32_t>(__double2loint(x));
+  return __uint_as_float(((hi - 0x38000000u) << 3) | (lo >> 29));  // x > 0
+}
+__device__ __forceinline__ double double_of(float x) {  // x > 0
+  const uint32_t b = __float_as_uint(x);
+  return __hiloint2double(static_cast<int>((b >> 3) + 0x38000000u), static_cast<int>(b << 29));
+}
+__device__ __forceinline__ double half_of(double x) {  // x / 2, x normal
+  return __hiloint2double(__double2hiint(x) - 0x100000, __double2loint(x));
+}
+
+// Householder scalars in binary64 with few instructions of its unit (17 with
+// the caller's s2; a square root and two divisions take over 40): r = 1/sqrt(s2)
+// by one Newton step from a binary32 seed (2^-22 -> 2^-43), the root s2 r and r
+// itself by a step each from there (quadratic: below an ulp), and 1/(|alpha| +
+// root) by the cubic step y (1 + e + e^2), e = 1 - d y (2^-22 -> 2^-66).
+// Outside the binary32 range the library's functions.
+static __device__ __noinline__ void make_reflector_slow(double s2, double alpha, Reflector<double>* f) {
+  *f = make_reflector(s2, alpha);
+}
+__device__ __forceinline__ Reflector<double> make_reflector64(double s2, double alpha) {
+  Reflector<double> f;
+  // 2^-113 <= s2 < 2^113 (integer test: no binary64 instruction)
+  if (static_cast<uint32_t>(__double2hiint(s2) >> 20) - 910u >= 226u) {
+    make_reflector_slow(s2, alpha, &f);
+    return f;
+  }
+  double r = double_of(rsqrtf(float_of(s2)));
+  r = fma(r, fma(-half_of(s2) * r, r, 0.5), r);
+  double sg = s2 * r;
+  sg = fma(fma(-sg, sg, s2), half_of(r), sg);
+  r = fma(fma(-sg, r, 1.0), r, r);
+  const double d = fabs(alpha) + sg;  // |alpha - beta|
+  double y = double_of(__frcp_rn(float_of(d)));
+  const double e = fma(-d, y, 1.0);
+  y = fma(fma(e, e, e), y, y);
+  f.beta = -copysign(sg, alpha);
+  f.scal = copysign(y, alpha);
+  f.ib = -copysign(r, alpha);
+  f.tau = d * r;  // (beta - alpha) / beta
+  f.ident = false;
+  return f;
+}
+
+// The column loops' reflector in the compute type.
+template <class T>
+__device__ __forceinline__ Reflector<T> column_reflector(T Sj, T alpha) {
+  if constexpr (std::is_same<T, double>::value) return make_reflector64(Sj, alpha);
+  else return make_reflector(Sj, alpha);
+}
 template <class T>
 __device__ __forceinline__ T shfl_from(T v, int src) {
   if constexpr (std::is_same<T, df64>::value) {
@@ -315,7 +368,7 @@ __device__ __forceinline__ void tile_update_la_x(T (&a)[R][NPC], const T (&d)[NP
 #pragma unroll
       for (int q = 0; q < 4; ++q)
         if (rbase + 32 * q == j + 1) al = a[q][C0];
-      const Reflector<T> f = make_reflector(ss, shfl_from(al, (j + 1) & 31));
+      const Reflector<T> f = column_reflector(ss, shfl_from(al, (j + 1) & 31));
       if ((threadIdx.x & 31) == 0) {
         refl_next[0] = f.beta;
         refl_next[1] = f.scal;
@@ -391,7 +444,7 @@ using YStore = typename std::conditional<std::is_same<T, df64>::value, df64, S>:
 // products that only give Gram entries (about a third of the column loop's
 // FMAs) are skipped; R is the same bit for bit.  With Y == NULL this is the
 // R-only form; with Y, the vectors and tau are written and the Gram entries
-// are left to k_gram_oz (the tensor-core Gram of the Ozaki form).
+// are left to k_gram_split.
 // Launch: blockDim = 32*CS*NRG <= MAXT, gridDim = p, dynamic smem = LocalQrSmem.
 // ---------------------------------------------------------------------------
 template <class S, class T, int NPC, int R, int MAXT, bool LA, bool GRAM = true>
@@ -504,7 +557,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_local_qr(const S* __restrict__ A, i
       if (LA) {
         // one row group: reflector 0 is formed here (the look-ahead loop
         // below has no barrier for column 0)
-        const Reflector<T> f0 = make_reflector(ss, shfl_from(a[0][0], 0));
+        const Reflector<T> f0 = column_reflector(ss, shfl_from(a[0][0], 0));
         if (lane == 0) {
           refl[0] = f0.beta;
           refl[1] = f0.scal;
@@ -575,14 +628,23 @@ __global__ void __launch_bounds__(MAXT, 1) k_local_qr(const S* __restrict__ A, i
           if constexpr (kXr) return xv[q];
           else return xcur[rbase + 32 * q];
         };
-        {
+        if constexpr (GRAM) {
           T s[NPC];
-          if constexpr (GRAM) {
-            column_dots_x(a, xr, s);
-          } else {
-            with_c0<NPC>(c0, [&](auto ic) { column_dots_from_x<decltype(ic)::value, NPC, R, T>(a, xr, s); });
-          }
+          column_dots_x(a, xr, s);
           TransposeReduce<NPC, 16>::run(s, lane, 0, NPC, rcur + warp * 32);
+        } else {
+          // the trailing columns only, in the warp sums too (each column's sum
+          // is the same tree of lanes for any number of columns)
+          with_c0<NPC>(c0, [&](auto ic) {
+            constexpr int C0 = decltype(ic)::value;
+            if constexpr (C0 < NPC) {
+              T s[NPC], v[NPC - C0];
+              column_dots_from_x<C0, NPC, R, T>(a, xr, s);
+#pragma unroll
+              for (int c = C0; c < NPC; ++c) v[c - C0] = s[c];
+              TransposeReduce<NPC - C0, 16>::run(v, lane, 0, NPC - C0, rcur + warp * 32 + C0);
+            }
+          });
         }
         __syncwarp();
 
@@ -680,7 +742,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_local_qr(const S* __restrict__ A, i
           if (lane == 0) {
             T Sj = T(0);
             for (int g = 0; g < NRG; ++g) Sj += ncur[g];
-            f = make_reflector(Sj, pcur[j]);
+            f = column_reflector(Sj, pcur[j]);
             refl[0] = f.beta;
             refl[1] = f.scal;
             refl[2] = f.ib;
@@ -785,7 +847,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_local_qr(const S* __restrict__ A, i
       //      form, binary64, into the upper triangle of the tile's T slot (the
       //      strictly lower part is never read); k_build_t turns them into T.
       //      Without the Gram dot products (GRAM = false) only tau_j is
-      //      written: the Gram entries come from k_gram_oz.
+      //      written: the Gram entries come from k_gram_split.
       {
         double* Tout = Tst + (static_cast<int64_t>(blockIdx.x) * kt + t) * n * n;
         if constexpr (GRAM) {
@@ -863,7 +925,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_local_qr(const S* __restrict__ A, i
 // tile, last to first, with X = C: tile t >= 1 has Householder vectors
 // [I; V_t], so W_t = T_t X, its rows of Q are -V_t W_t and tile t-1 gets
 // X - W_t; tile 0 is the one-tile case with C = X.
-//   Yg  : m x n (storage S), as written by k_local_qr.
+//   Yg  : m x n (storage S), as written by Step 1 (tiles of B, then bt rows).
 //   Tg  : kt slots of n x n binary64 per block (T of each tile, upper part).
 //   Cg  : cblocks blocks of n x n binary64 (cblocks == 1: one C for all).
 //   Qg  : output m x n (storage S); may alias Yg.
@@ -878,14 +940,13 @@ template <int NPC>
 constexpr int max_entries() { return (NPC * 100 + 31) / 32; }  // n <= 100
 
 template <class S, class T, int NPC, int R, int MAXT>
-__global__ void __launch_bounds__(MAXT, 1) k_form_q(const S* Yg, int64_t m, int n, int b, int bt, int kt, int srows,
+__global__ void __launch_bounds__(MAXT, 1) k_form_q(const S* Yg, int64_t m, int n, int b, int B, int bt, int kt, int srows,
                                                      int CS, int NRG, int skew, const double* __restrict__ Tg,
                                                      const double* __restrict__ Cg, int64_t cblocks, S* Qg,
                                                      int32_t* status) {
   extern __shared__ __align__(128) unsigned char smem[];
   const int NT = blockDim.x;
   const int NPAD = NPC * CS;
-  const int B = 32 * NRG * R;
   const FormQSmem L(srows, n, NPAD, sizeof(S), sizeof(T));
   S* stage = reinterpret_cast<S*>(smem + L.stage);
   T* Xm = reinterpret_cast<T*>(smem + L.xm);

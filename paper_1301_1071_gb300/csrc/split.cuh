@@ -37,6 +37,14 @@ __device__ __forceinline__ void mma_f16(float (&d)[4], uint32_t a0, uint32_t a1,
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
+// The same with its own addend: D = A B + (c, c, c, c).
+__device__ __forceinline__ void mma_f16_c(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                          uint32_t b0, uint32_t b1, float c) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(c));
+}
+
 constexpr int kExpZero = -100000;  // "exponent" of a zero entry in a maximum
 constexpr int kExpBad = 1 << 20;   // ... of a column of M with Inf or NaN
 
@@ -93,17 +101,25 @@ __device__ __forceinline__ int split_int(float acc) {
   return static_cast<int>(__float_as_uint(acc) - kSplitMagicBits);
 }
 
-// P 2^s rounded to nearest (ties up in magnitude) with integer operations.
+// P 2^s rounded to nearest (ties up in magnitude) with integer operations;
+// outside the normal range (and for zero) by a call.
+static __device__ __noinline__ double split_to_double_slow(long long P, int s) {
+  return P == 0 ? 0.0 : ldexp(static_cast<double>(P), s);
+}
 __device__ __forceinline__ double split_to_double(long long P, int s) {
+  const uint32_t sign = static_cast<uint32_t>(static_cast<unsigned long long>(P) >> 32) & 0x80000000u;
   const unsigned long long u = static_cast<unsigned long long>(P < 0 ? -P : P);
   const int lz = __clzll(static_cast<long long>(u));
-  const unsigned long long w = u << lz;                       // bit 63 set (u != 0)
-  const unsigned long long r = (w >> 11) + ((w >> 10) & 1ull);  // 53 bits, or 2^53
-  const int e = s + 63 - lz + 1022;  // biased exponent less one: r's hidden bit adds it
-  if (u == 0ull) return 0.0;
-  if (e < 0 || e > 2044) return ldexp(static_cast<double>(P), s);
-  const unsigned long long bits = (static_cast<unsigned long long>(e) << 52) + r;
-  return __longlong_as_double(static_cast<long long>(P < 0 ? bits | (1ull << 63) : bits));
+  const unsigned long long w = (u << lz) + 0x400ull;  // bit 63 set; a carry out means 2^64
+  // the significand's 53 bits (its hidden bit adds one to the exponent field);
+  // a carry out of the rounding leaves w near 0: the exponent takes it
+  const uint32_t wl = static_cast<uint32_t>(w), wh = static_cast<uint32_t>(w >> 32);
+  const bool carry = wh < 0x80000000u;
+  const int e = s - lz + (carry ? 1086 : 1085);  // biased exponent less one
+  if (static_cast<uint32_t>(e) > 2044u || u == 0ull) return split_to_double_slow(P, s);
+  const uint32_t mh = (carry ? 0x100000u : (wh >> 11));
+  const uint32_t ml = __funnelshift_r(wl, wh, 11);
+  return __hiloint2double(static_cast<int>((static_cast<uint32_t>(e) << 20) + mh | sign), static_cast<int>(ml));
 }
 
 // sum_D v_D 2^(44 - 8 D), D = 0 .. 7 (the last two rounded): the digit

@@ -270,15 +270,17 @@ __global__ void __launch_bounds__(kRsThreads, KC <= 2 ? 2 : 1)
             if (r < n && c < n) {
               double v = split_to_double(o[i], er[i >> 1] + cexp[c] - kSplitShift);
               if (bad[i >> 1] || cexp[c] == kExpBad) v = __longlong_as_double(0x7ff8000000000000ll);
-              wm[r * n + c] = fma(Tb[static_cast<int64_t>(r) * n + r], src[r * n + c], v);
+              const double tau = Tb[static_cast<int64_t>(r) * n + r], xo = src[r * n + c];
+              wm[r * n + c] = fma(tau, xo, v);
+              // the coefficient of tile t - 1, X - W = -X + ((2 - tau) X - v):
+              // with tau close to 2 one rounding of X a tile
+              if (!top) xm[r * n + c] = fma(2.0 - tau, xo, -v) - xo;
             }
           }
         }
       }
     }
     __syncthreads();
-    if (!top)
-      for (int e = threadIdx.x; e < nn; e += kRsThreads) xm[e] -= wm[e];  // coefficient of tile t - 1
     split_build_b([&](int k, int c) { return wm[k * n + c]; }, n, KC, nullptr, cexp, bfrag);
     __syncthreads();
     for (int p0 = warp * kRsRows; p0 < cnt; p0 += kRsRows * NWARP) {

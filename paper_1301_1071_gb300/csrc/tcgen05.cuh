@@ -53,23 +53,6 @@ __device__ __forceinline__ void tc_commit(uint64_t* bar) {
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// tcgen05.mma kind::f16 with binary16 A and B (same type) and a binary32
-// accumulator in tensor memory.
-__device__ __forceinline__ void tc_mma_f16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, int acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc)
-      : "memory");
-}
-
-// Instruction descriptor of kind::f16: binary32 accumulator (bits 4-5 = 1),
-// A and B binary16 (bits 7-9 and 10-12 = 0), both K-major, N >> 3 at bit 17,
-// M >> 4 at bit 24.
-__host__ __device__ constexpr uint32_t tc_idesc_f16(int M, int N) {
-  return (1u << 4) | (static_cast<uint32_t>(N >> 3) << 17) | (static_cast<uint32_t>(M >> 4) << 24);
-}
-
 // 8 consecutive 32-bit columns of this warp's 32 tensor-memory lanes (one
 // row per lane), completed by tc_wait_ld.
 __device__ __forceinline__ void tc_ld_x8(uint32_t taddr, uint32_t (&v)[8]) {
