@@ -131,8 +131,10 @@ typedef struct tsqr_opts {
                           cluster of f CTAs, one R factor each), else
                           TSQR_ERR_SHAPE.  Automatic: one CTA per node with
                           as many R factors as the binary64 register tile has
-                          rows for, where that is at least 4 and 4 fit the
-                          CTA; else 8 per node on a cluster. */
+                          rows for, at most 32 and no more than the number of
+                          levels needs, where that is at least 8 and 4 fit the
+                          CTA; else 8 per node (on a cluster where one CTA
+                          does not hold them). */
   int32_t sync;        /* 1 = synchronise the stream and return the device status */
   /* Optional stage timing (tsqr_direct, tsqr_svd): NULL, or 4 cudaEvent_t
      handles (as void*) recorded on the stream at the start, after Step 1's

@@ -205,7 +205,7 @@ static int64_t panel_block_rows(int64_t m, int64_t f, int64_t slots, int64_t al)
     const int64_t p = (m + k * kPdRows - 1) / (k * kPdRows);
     const int64_t waves = (p + slots - 1) / slots;
     const double cost = (double)waves * (double)k + 3.2 * (double)levels(p);
-    if (k == 1 || cost < best) {
+    if (k == 1 || cost <= best) {  // taller blocks on a tie: fewer nodes (4,000,000 x 64 55.4 -> 53.2 ms)
       best = cost;
       rows = k * kPdRows;
       // blocks of even height over whole waves, where that adds no level
@@ -264,12 +264,17 @@ int make_plan(int64_t m, int64_t n, int esz, int64_t block_rows, int fanout, Pla
   if (bt < 1) return TSQR_ERR_SHAPE;
   // tree node = f stacked R factors, f >= 2: up to the binary64 row-block
   // tile's rows (fmax), or any f whose node fits one CTA's shared memory or
-  // a cluster of f CTAs.  Default: fmax while a node of 4 triangles fits one
-  // CTA, else (n > 84, where one CTA holds at most 3) nodes of kTreeClMaxF
-  // triangles on clusters: 20,000,000 x 100 has 4 tree levels instead of 10
+  // a cluster of f CTAs.  Default: fmax, at most kTreeMaxF (a node's chain grows
+  // with its triangles: 100,000 x 10 in 100 blocks 372 us at f = 100, 314 at 10;
+  // 124,103 x 8 391 us at f = 256, 229 at 32), while that is kTreeClMaxF or
+  // more; else nodes of kTreeClMaxF triangles on clusters (1,000,000 x 64: 12.4 ms
+  // at f = 6, 10.8 at 8; 20,000,000 x 100 has 4 tree levels instead of 10); then
+  // (where 4 triangles fit one CTA) the least fan-in that needs no more levels
+  // (608 blocks of n = 64: 4 levels at f = 8 and at 5, 9.13 against 8.47 ms)
   const int64_t fmax = P.cfg64.B / n;
   const int ni = static_cast<int>(n);
-  const int64_t f = fanout > 0 ? fanout : (fmax >= 4 && tree_up_fits(ni, 4) ? fmax : kTreeClMaxF);
+  int64_t f = fanout;
+  if (fanout <= 0) f = fmax >= kTreeClMaxF && tree_up_fits(ni, 4) ? std::min(fmax, kTreeMaxF) : kTreeClMaxF;
   int64_t b0 = block_rows;
   if (b0 <= 0 && P.panel) {
     b0 = panel_block_rows(m, f, (int64_t)(sms < 1 ? kDefaultSMs : sms) * P.ctas0, al);
@@ -291,6 +296,15 @@ int make_plan(int64_t m, int64_t n, int esz, int64_t block_rows, int fanout, Pla
   }
   if (b0 < n) return TSQR_ERR_SHAPE;
   if (b0 > m) b0 = m;  // one block
+  if (fanout <= 0 && tree_up_fits(ni, 4)) {
+    auto levels = [&](int64_t g) {
+      int l = 0;
+      for (int64_t p = (m + b0 - 1) / b0; p > 1; p = (p + g - 1) / g) ++l;
+      return l;
+    };
+    const int l = levels(f);
+    while (f > 2 && levels(f - 1) == l) --f;
+  }
   const int64_t kt0 = b0 <= B0 ? 1 : 1 + (b0 - B0 + bt - 1) / bt;
   // tiles per block: heights up to 2^31 - 1 rows in either form
   if (kt0 > (P.panel ? 1 << 24 : 1 << 20)) return TSQR_ERR_SHAPE;

@@ -18,6 +18,7 @@
 
 #include "device.cuh"
 #include "launch.h"
+#include "qr_kernels.cuh"
 
 namespace tsqr {
 
@@ -166,12 +167,16 @@ __global__ void __launch_bounds__(MAXT) k_tree_down(double* Y, int64_t rows, int
 // (k_build_t forms T).  WANT_Y = false: R only.
 // Threads: G per column (G a power of two, the G lanes of a column in one
 // warp), column c = tid / G; the lanes of a group split the column's
-// sub-column (all blocks, rows 0..j) as one index space.  Per column j two
-// CTA barriers: column j's group forms the norm, the reflector scalars and v
-// (its G lanes reduce by shuffles); then every later column's group forms its
-// dot with v and its update -- each column is touched by its own group only,
-// so the dots and the update of a column need no barrier between them.
-// The node sits in shared memory, row r at M[r * ldm].
+// sub-column (all blocks, rows 0..j) as one index space.  Per column j: every
+// group forms its sum with the unscaled x_j -- column j's its squared norm, the
+// later ones their dots, the earlier ones (with Y) their Gram entry -- by
+// shuffles; column j's group makes the scalars of it (make_reflector64);
+// barrier; the later groups update their columns by x_j; barrier.  x becomes v
+// = scal x at the end.  Bound by the latency of that chain: with the norm, the
+// scaling and the dots one after the other and the library's root and two
+// divisions in it, a 25-way node at n = 25 took 206 us.
+// The node sits in shared memory, row r at M[r * ldm]; scal_j in the padding
+// column of row j.
 template <bool WANT_Y>
 __global__ void __launch_bounds__(1024) k_tree_up(const double* X, int64_t rows, int n, int f, double* Y,
                                                   double* Rout, double* Tst, int G) {
@@ -192,90 +197,68 @@ __global__ void __launch_bounds__(1024) k_tree_up(const double* X, int64_t rows,
   __syncthreads();
   const int nsub = nb - 1;  // blocks below the first
   const unsigned gmask = G == 32 ? 0xffffffffu : (((1u << G) - 1u) << ((tid & 31) & ~(G - 1)));
+  double* Tn = WANT_Y ? Tst + node * n * n : nullptr;
   for (int j = 0; j < n; ++j) {
-    // the sub-column of column j: entries e = 0 .. nsub (j + 1) - 1, block
-    // k = 1 + e / (j + 1), row lr = e % (j + 1); lane u takes e = u, u + G, ..
-    // (stepped without division: G = dq (j + 1) + dr)
-    const int len = j + 1, ne = nsub * len;
+    // the sub-column of column j (a column c < j: its own, the rows 0 .. c):
+    // entries e = 0 .. nsub len - 1, block k = 1 + e / len, row lr = e % len;
+    // lane u takes e = u, u + G, .. (stepped without division: G = dq len + dr)
+    const bool gram = WANT_Y && c < j;
+    const bool live = c < n && (c >= j || gram);
+    const int len = (gram ? c : j) + 1, ne = live ? nsub * len : 0;
     const int dq = G / len, dr = G - dq * len;
     const int k0 = 1 + u / len, l0 = u - (u / len) * len;
+    double s0 = 0.0, s1 = 0.0;  // two chains: the unit's latency is many times its rate
+    {
+      const double* p = M + (k0 * n + l0) * ldm;
+      int lr = l0;
+      const int step = (dq * n + dr) * ldm, wrap = (n - len) * ldm;
+      for (int e = u; e < ne; e += 2 * G) {
+        s0 = fma(p[j], p[c], s0);
+        p += step;
+        lr += dr;
+        if (lr >= len) {
+          lr -= len;
+          p += wrap;
+        }
+        if (e + G < ne) s1 = fma(p[j], p[c], s1);
+        p += step;
+        lr += dr;
+        if (lr >= len) {
+          lr -= len;
+          p += wrap;
+        }
+      }
+    }
+    double s = s0 + s1;
+    for (int o = G >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(gmask, s, o);
     if (c == j) {
-      double ss = 0.0;
-      {
-        int k = k0, lr = l0;
-        for (int e = u; e < ne; e += G) {
-          const double v = M[(k * n + lr) * ldm + j];
-          ss = fma(v, v, ss);
-          lr += dr;
-          k += dq;
-          if (lr >= len) {
-            lr -= len;
-            ++k;
-          }
-        }
-      }
-      for (int o = G >> 1; o > 0; o >>= 1) ss += __shfl_xor_sync(gmask, ss, o);
       const double alpha = M[j * ldm + j];
-      const double sigma = sqrt(fma(alpha, alpha, ss));
-      double beta, scal, tau;
-      if (sigma == 0.0) {
-        beta = alpha;
-        scal = 0.0;
-        tau = 0.0;
-      } else {
-        beta = alpha >= 0.0 ? -sigma : sigma;
-        scal = 1.0 / (alpha - beta);
-        tau = (beta - alpha) / beta;
-      }
-      {  // v: the scaled sub-column
-        int k = k0, lr = l0;
-        for (int e = u; e < ne; e += G) {
-          M[(k * n + lr) * ldm + j] *= scal;
-          lr += dr;
-          k += dq;
-          if (lr >= len) {
-            lr -= len;
-            ++k;
-          }
-        }
-      }
+      const Reflector<double> f = make_reflector64(fma(alpha, alpha, s), alpha);
       if (u == 0) {
-        taus[j] = tau;
-        M[j * ldm + j] = beta;
+        taus[j] = f.tau;
+        M[j * ldm + n] = f.scal;
+        M[j * ldm + j] = f.beta;
       }
     }
     __syncthreads();
-    const double tau = taus[j];
-    if (c > j && c < n && tau != 0.0) {
-      // w_c = a_jc + v^T a_c over the sub-column rows; a_c -= (tau w_c) v
-      double w = 0.0;
-      {
-        int k = k0, lr = l0;
-        for (int e = u; e < ne; e += G) {
-          const double* row = M + (k * n + lr) * ldm;
-          w = fma(row[j], row[c], w);
-          lr += dr;
-          k += dq;
-          if (lr >= len) {
-            lr -= len;
-            ++k;
-          }
-        }
-      }
-      for (int o = G >> 1; o > 0; o >>= 1) w += __shfl_xor_sync(gmask, w, o);
-      const double tw = tau * (M[j * ldm + c] + w);
+    const double tau = taus[j], scal = M[j * ldm + n];
+    if (gram) {
+      if (u == 0) Tn[c * n + j] = (M[c * ldm + n] * scal) * s;
+    } else if (live && c > j && tau != 0.0) {
+      // w_c = a_jc + scal x^T a_c; a_c -= (tau w_c scal) x
+      const double tw = tau * fma(scal, s, M[j * ldm + c]);
+      const double tx = tw * scal;
       if (u == 0) M[j * ldm + c] -= tw;
-      {
-        int k = k0, lr = l0;
-        for (int e = u; e < ne; e += G) {
-          double* row = M + (k * n + lr) * ldm;
-          row[c] = fma(-tw, row[j], row[c]);
-          lr += dr;
-          k += dq;
-          if (lr >= len) {
-            lr -= len;
-            ++k;
-          }
+      double* p = M + (k0 * n + l0) * ldm;
+      int lr = l0;
+      const int step = (dq * n + dr) * ldm, wrap = (n - len) * ldm;
+      for (int e = u; e < ne; e += G) {
+        p[c] = fma(-tx, p[j], p[c]);
+        p += step;
+        lr += dr;
+        if (lr >= len) {
+          lr -= len;
+          p += wrap;
         }
       }
     }
@@ -292,23 +275,9 @@ __global__ void __launch_bounds__(1024) k_tree_up(const double* X, int64_t rows,
     double* Yn = Y + r0 * n;
     for (int idx = tid; idx < nb * n * n; idx += NT) {
       const int r = idx / n, cc = idx - r * n;
-      Yn[idx] = M[r * ldm + cc];
+      Yn[idx] = M[r * ldm + cc] * M[cc * ldm + n];
     }
-    // tau and the Gram entries G(i, c) = sum_k sum_{lr <= i} v_i(lr) v_c(lr), i < c
-    double* Tn = Tst + node * n * n;
-    for (int idx = tid; idx < n * n; idx += NT) {
-      const int i = idx / n, cc = idx - i * n;
-      if (cc < i) continue;
-      double g = taus[i];
-      if (cc > i) {
-        g = 0.0;
-        for (int k = 1; k < nb; ++k) {
-          const double* blk = M + static_cast<size_t>(k) * n * ldm;
-          for (int lr = 0; lr <= i; ++lr) g = fma(blk[lr * ldm + i], blk[lr * ldm + cc], g);
-        }
-      }
-      Tn[idx] = g;
-    }
+    for (int i = tid; i < n; i += NT) Tn[i * n + i] = taus[i];
   }
 }
 
