@@ -61,6 +61,8 @@ cudaError_t launch_gram(int esz, const void* X, const void* Y, int64_t m, int n,
                               colexp, st)
       : esz == 8
           ? launch_gram_f64(X, Y, m, n, g.chunk, g.grid, g.nt, g.tile, acc_storage, part, status, st)
+      : !acc_storage && X == Y && n >= kGramSplitF32MinN
+          ? launch_gram_split_f32(static_cast<const float*>(X), m, n, g.grid, &parts, part, st)
           : launch_gram_f32(X, Y, m, n, g.chunk, g.grid, g.nt, g.tile, acc_storage, part, status, st);
   if (e != cudaSuccess) return e;
   return launch_gram_reduce(part, parts, n, G, status, st);
@@ -110,7 +112,10 @@ cudaError_t launch_form_q(const KernelCfg& k, const void* Y, int64_t m, int n, i
                           cudaStream_t st) {
   switch (k.kind) {
     case kKindF64: return launch_form_q_f64(k, Y, m, n, b, B, bt, kt, p, T, C, cblocks, Q, status, st);
-    case kKindF32: return launch_form_q_f32(k, Y, m, n, b, B, bt, kt, p, T, C, cblocks, Q, status, st);
+    case kKindF32:
+      if (step3_rows32(n) && Y == Q)
+        return launch_form_q_f32_tiles(static_cast<float*>(Q), m, n, b, B, bt, kt, p, T, C, cblocks, st);
+      return launch_form_q_f32(k, Y, m, n, b, B, bt, kt, p, T, C, cblocks, Q, status, st);
     case kKindDF64: return launch_form_q_df64(k, Y, m, n, b, B, bt, kt, p, T, C, cblocks, Q, status, st);
     default: return cudaErrorInvalidValue;
   }
@@ -391,9 +396,14 @@ tsqr_status run_r_only(const Plan& P, int esz, const void* X, double* R, void* w
 tsqr_status rowmul(const Plan& P, const void* X, const double* M1, const void* Y, const double* M2, void* out,
                    int32_t* status, cudaStream_t st, const double* xsrc = nullptr, const int* xexp = nullptr) {
   const int ni = static_cast<int>(P.n);
+  const size_t bytes = static_cast<size_t>(P.m) * P.n * P.esz;
+  auto clash = [&](const void* in) { return in && in != out && overlaps(in, bytes, out, bytes); };
+  if (P.esz == 4 && ni >= kRows32MinN && !clash(X) && !clash(Y)) {
+    TSQR_CUDA(launch_rowmul_f32_tiles(static_cast<const float*>(X), M1, static_cast<const float*>(Y), M2, P.m, ni,
+                                      static_cast<float*>(out), st));
+    return TSQR_OK;
+  }
   if (P.esz == 8 && rows_by_digits(ni)) {
-    const size_t bytes = static_cast<size_t>(P.m) * P.n * 8;
-    auto clash = [&](const void* in) { return in && in != out && overlaps(in, bytes, out, bytes); };
     if (!clash(X) && !clash(Y) && !(X == out && Y == out)) {
       const double *x = static_cast<const double*>(X), *y = static_cast<const double*>(Y);
       double* o = static_cast<double*>(out);

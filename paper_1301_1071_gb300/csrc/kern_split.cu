@@ -44,14 +44,14 @@ cudaError_t launch_form_q_split(double* Y, int64_t m, int n, int64_t b, int B, i
 // Tiles per warp: ncg warps share the output tiles of ncg (and ncg / 2)
 // column groups; 64-row chunks for n <= 64, 32-row chunks above (the digit
 // planes of both operands then fit an SM).
-template <bool SYM, bool TM>
-static cudaError_t gram_split(const double* X, const double* Y, int64_t m, int n, double* part, int* colexp, int64_t b,
+template <class S, bool SYM, bool TM>
+static cudaError_t gram_split(const S* X, const S* Y, int64_t m, int n, double* part, int* colexp, int64_t b,
                               int B, int bt, int kt, int64_t p, int64_t work, int64_t* grid_max, cudaStream_t st) {
   const int ncg = (n + 7) / 8;
   const int CR = n <= 64 ? 64 : 32;
-  auto fn = n <= 32   ? k_gram_split<SYM, TM, 64, 2, 128, SYM ? 3 : 2>
-            : n <= 64 ? k_gram_split<SYM, TM, 64, SYM ? 3 : 4, 256, 1>
-                      : k_gram_split<SYM, TM, 32, SYM ? 4 : 7, 416, 1>;
+  auto fn = n <= 32   ? k_gram_split<S, SYM, TM, 64, 2, 128, SYM ? 3 : 2>
+            : n <= 64 ? k_gram_split<S, SYM, TM, 64, SYM ? 3 : 4, 256, 1>
+                      : k_gram_split<S, SYM, TM, 32, SYM ? 4 : 7, 416, 1>;
   const size_t smem = GramSplitSmem(n, CR, SYM).total;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
@@ -73,8 +73,19 @@ cudaError_t launch_gram_split(const double* X, const double* Y, int64_t m, int n
   const int CR = n <= 64 ? 64 : 32;
   const int64_t chunks = (m + CR - 1) / CR;
   int64_t grid = max_parts;
-  const cudaError_t e = X == Y ? gram_split<true, false>(X, X, m, n, part, colexp, 0, 0, 0, 1, 0, chunks, &grid, st)
-                               : gram_split<false, false>(X, Y, m, n, part, colexp, 0, 0, 0, 1, 0, chunks, &grid, st);
+  const cudaError_t e = X == Y ? gram_split<double, true, false>(X, X, m, n, part, colexp, 0, 0, 0, 1, 0, chunks, &grid, st)
+                               : gram_split<double, false, false>(X, Y, m, n, part, colexp, 0, 0, 0, 1, 0, chunks, &grid, st);
+  *parts = static_cast<int>(grid);
+  return e;
+}
+
+cudaError_t launch_gram_split_f32(const float* X, int64_t m, int n, int max_parts, int* parts, double* part,
+                                  cudaStream_t st) {
+  if (n < 1 || n > TSQR_NMAX) return cudaErrorInvalidValue;
+  const int CR = n <= 64 ? 64 : 32;
+  int64_t grid = max_parts;
+  const cudaError_t e =
+      gram_split<float, true, false>(X, X, m, n, part, nullptr, 0, 0, 0, 1, 0, (m + CR - 1) / CR, &grid, st);
   *parts = static_cast<int>(grid);
   return e;
 }
@@ -83,7 +94,7 @@ cudaError_t launch_gram_t_split(const double* Y, int64_t m, int n, int64_t b, in
                                 double* T, cudaStream_t st) {
   if (n < 1 || n > TSQR_NMAX) return cudaErrorInvalidValue;
   int64_t grid = 1 << 30;
-  return gram_split<true, true>(Y, Y, m, n, T, nullptr, b, B, static_cast<int>(bt), kt, p, p * kt, &grid, st);
+  return gram_split<double, true, true>(Y, Y, m, n, T, nullptr, b, B, static_cast<int>(bt), kt, p, p * kt, &grid, st);
 }
 
 }  // namespace tsqr

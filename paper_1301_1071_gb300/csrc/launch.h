@@ -83,10 +83,30 @@ cudaError_t launch_form_q_split(double* Y, int64_t m, int n, int64_t b, int B, i
 // exponents of X's columns.
 cudaError_t launch_gram_split(const double* X, const double* Y, int64_t m, int n, int max_parts, int* parts,
                               double* part, int* colexp, cudaStream_t st);
+// X^T X of binary32 data with binary64 accuracy (Cholesky QR), n >=
+// kGramSplitF32MinN: below, binary64 FMAs take no longer (Cholesky QR of
+// 3,000,000 x 9: 1.73 ms by FMAs, 2.15 by digits; x 12: 2.71 and 1.49).
+constexpr int kGramSplitF32MinN = 12;
+cudaError_t launch_gram_split_f32(const float* X, int64_t m, int n, int max_parts, int* parts, double* part,
+                                  cudaStream_t st);
 // The Gram entries of every tile's Householder vectors into the T slots'
 // strictly upper triangles.
 cudaError_t launch_gram_t_split(const double* Y, int64_t m, int n, int64_t b, int B, int64_t bt, int kt, int64_t p,
                                 double* T, cudaStream_t st);
+
+// binary32 row products in 128-row tiles (rows32.cuh), n >= kRows32MinN:
+// out = X M1 + Y M2 (either input NULL; out may be an input), and Step 3 in
+// binary32 arithmetic (Q over Y).  Below n = 8 a thread's 8 columns are padding
+// in part (4,000,000 x 8, Step 1, 3 and adjoint: 1.37 -> 1.15 ms).  Step 3 with
+// odd n > 64 keeps k_form_q: rows copied 4 bytes at a time, and two tiles and
+// two matrices leave one CTA an SM (2,000,000 x 77 with adjoint 16.5 ms there,
+// 16.8 here; x 98 27.2 there, 25.0 here).
+constexpr int kRows32MinN = 8;
+constexpr bool step3_rows32(int n) { return n >= kRows32MinN && (n <= 64 || n % 2 == 0); }
+cudaError_t launch_rowmul_f32_tiles(const float* X, const double* M1, const float* Y, const double* M2, int64_t m,
+                                    int n, float* out, cudaStream_t st);
+cudaError_t launch_form_q_f32_tiles(float* Y, int64_t m, int n, int64_t b, int B, int64_t bt, int kt, int64_t p,
+                                    const double* T, const double* C, int64_t cblocks, cudaStream_t st);
 
 // Gram launch geometry shared by the planner and the launcher.
 struct GramGeom { int chunk, grid, nt, tile; };

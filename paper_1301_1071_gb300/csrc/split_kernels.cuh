@@ -3,6 +3,7 @@
 #pragma once
 
 #include <cstdint>
+#include <type_traits>
 
 #include "device.cuh"
 #include "layout.cuh"
@@ -366,9 +367,9 @@ struct GramSplitSmem {
   }
 };
 
-template <bool SYM, bool TM, int CR, int TW, int MAXT, int MINB>
+template <class S, bool SYM, bool TM, int CR, int TW, int MAXT, int MINB>
 __global__ void __launch_bounds__(MAXT, MINB)
-    k_gram_split(const double* __restrict__ X, const double* __restrict__ Yin, int64_t m, int n, double* part,
+    k_gram_split(const S* __restrict__ X, const S* __restrict__ Yin, int64_t m, int n, double* part,
                  int* colexp, int64_t b, int B, int bt, int kt, int64_t p) {
   static_assert(!TM || SYM, "the T factors' Gram is symmetric");
   extern __shared__ __align__(128) unsigned char smem[];
@@ -390,16 +391,17 @@ __global__ void __launch_bounds__(MAXT, MINB)
   __syncthreads();
 
   const int c0 = 8 * warp + 2 * t;  // this lane's column pair in the loads
-  const bool wide = (n & 1) == 0;   // rows start on 16-byte boundaries
-  auto load = [&](const double* S, int64_t r0, int rows, double (&v)[RL][2], int top) {
+  const bool wide = (n & 1) == 0;   // pairs of entries are aligned
+  using S2 = typename std::conditional<sizeof(S) == 8, double2, float2>::type;
+  auto load = [&](const S* src, int64_t r0, int rows, double (&v)[RL][2], int top) {
 #pragma unroll
     for (int i = 0; i < RL; ++i) {
       const int r = 8 * i + g;
       v[i][0] = v[i][1] = 0.0;
       if (r < rows && c0 < n) {
-        const double* q = S + (r0 + r) * n + c0;
+        const S* q = src + (r0 + r) * n + c0;
         if (wide) {
-          const double2 w = *reinterpret_cast<const double2*>(q);
+          const S2 w = *reinterpret_cast<const S2*>(q);
           v[i][0] = w.x;
           v[i][1] = w.y;
         } else {

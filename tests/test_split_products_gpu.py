@@ -128,3 +128,73 @@ def test_non_finite_is_reported(value):
     with pytest.raises(T.TSQRError) as e:
         T.direct(_cuda(A))
     assert e.value.status == 8
+
+
+def _f32(a):
+    return torch.tensor(np.ascontiguousarray(a), dtype=torch.float32, device="cuda")
+
+
+# binary32: 8-column thread groups, k steps of 4, copies of 16, 8 or 4 bytes (n
+# mod 4), 128-row tiles.  A product entry is a chain of at most 2 n binary32
+# FMAs: 4 n 2^-24 of its row by column scale, and kappa of R for the adjoint.
+@pytest.mark.parametrize("n", [7, 8, 9, 11, 12, 25, 32, 33, 50, 63, 64, 65, 66, 77, 98, 100])
+@pytest.mark.parametrize("m,b", [(127, 0), (128, 0), (2003, 701)])
+def test_binary32_direct_edges(m, n, b):
+    A = ti.gaussian(m, n, 8).astype(np.float32)
+    Q, R = _T().direct(_f32(A), block_rows=b, prec="native")
+    Q, R = Q.double().cpu().numpy(), R.cpu().numpy()
+    Qo, Ro = oracle.householder_qr(A.astype(np.float64))
+    tol = 10 * n * np.linalg.cond(A) * 2.0 ** -24
+    assert np.linalg.norm(R - Ro) <= tol * np.linalg.norm(Ro)
+    assert np.max(np.abs(Q - Qo)) <= tol
+    assert oracle.orth_error(Q)[0] <= 1e-5
+
+
+@pytest.mark.parametrize("n", [7, 8, 9, 12, 25, 33, 50, 65, 98])
+@pytest.mark.parametrize("m", [127, 1003])
+def test_binary32_backward_edges(m, n):
+    A, dQ, dR = ti.gaussian(m, n, 1), ti.gaussian(m, n, 2).astype(np.float32), ti.gaussian(n, n, 3)
+    Qo, Ro = oracle.householder_qr(A)
+    Q32 = Qo.astype(np.float32)
+    got = _T().backward(_f32(Q32), _cuda(Ro), _f32(dQ), _cuda(dR)).double().cpu().numpy()
+    want = oracle.qr_backward(Q32.astype(np.float64), Ro, dQ.astype(np.float64), np.triu(dR))
+    tol = 4 * n * 2.0 ** -24 * np.linalg.cond(Ro)
+    assert np.linalg.norm(got - want) <= tol * np.linalg.norm(want)
+
+
+def test_binary32_backward_in_place():
+    T = _T()
+    m, n = 1003, 25
+    Qo, Ro = oracle.householder_qr(ti.gaussian(m, n, 1))
+    Q, R, dQ = _f32(Qo), _cuda(Ro), _f32(ti.gaussian(m, n, 2))
+    want = T.backward(Q, R, dQ, None)
+    lib = T.load()
+    need = T.workspace_size(T.OP_BACKWARD, m, n, torch.float32)
+    work = torch.empty(need, dtype=torch.uint8, device="cuda")
+    for over in ("dQ", "Q"):
+        q, d = Q.clone(), dQ.clone()
+        out = d if over == "dQ" else q
+        st = lib.tsqr_backward(ctypes.c_void_p(q.data_ptr()), ctypes.c_void_p(R.data_ptr()),
+                               ctypes.c_void_p(d.data_ptr()), None, m, n, 1, ctypes.c_void_p(out.data_ptr()),
+                               ctypes.c_void_p(work.data_ptr()), need, None,
+                               ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+        assert st == 0
+        torch.cuda.synchronize()
+        assert torch.equal(out, want), over  # the same sums in the same order
+
+
+@pytest.mark.parametrize("n", [7, 11, 12, 13, 25, 33, 50, 65, 100])
+def test_binary32_cholqr(n):
+    """The Gram of binary32 data is exact to binary64 rounding: R is the oracle's
+    to kappa^2 2^-52, Q to its storage."""
+    A = ti.column_scaled(4003, n, 1e-4, 4).astype(np.float32)
+    Q, R = _T().cholqr(_f32(A))
+    Qo, Ro = oracle.householder_qr(A.astype(np.float64))
+    kappa = np.linalg.cond(A / np.linalg.norm(A, axis=0)[None, :])
+    assert np.max(np.abs(Q.double().cpu().numpy() - Qo)) <= 10 * n * kappa ** 2 * 2.0 ** -24
+    # the second pass factors the binary32 Q, so R carries its rounding
+    assert np.max(np.linalg.norm(R.cpu().numpy() - Ro, axis=0) / np.linalg.norm(Ro, axis=0)) \
+        <= 10 * n * kappa ** 2 * 2.0 ** -24
+    A[77, 5] = np.inf
+    with pytest.raises(_T().TSQRError):
+        _T().cholqr(_f32(A))
