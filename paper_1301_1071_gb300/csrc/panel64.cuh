@@ -25,6 +25,11 @@
 // cores, with the digit index packed into the idle halves of the
 // fragments.  The running R stays in shared memory: tile t >= 1 factors
 // [R; A_t] with vectors [I; V_t].
+//
+// Measured: Step 1 of 4,000,000 x 64 65.2 -> 20.9 ms plus 3.2 for T's Gram (its
+// bytes 0.6; 2 m n^2 binary64 flops would take 27), 3,000,000 x 32 10.96 -> 5.68.
+// Bound by the chain of panels a tile runs through: the binary64 unit is 44 to
+// 57 % busy with conversions, the columns and T_p^T.
 #pragma once
 
 #include <cstdint>
@@ -245,8 +250,8 @@ __device__ __forceinline__ void panel64_factor(double (&a)[kPdRL][kPdCols], doub
 // instruction cache on every second fetch.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kPdMaxThreads, 1)
-    k_panel_qr_f64(const double* __restrict__ A, int64_t m, int n, int b, int kt, int NW, int NS, double* Y,
-                   double* __restrict__ Rst, double* __restrict__ Tst, int32_t* status) {
+    k_panel_qr_f64(const double* __restrict__ A, int64_t m, int n, int b, int kt, int NW, int NS, uint64_t order,
+                   double* Y, double* __restrict__ Rst, double* __restrict__ Tst, int32_t* status) {
   constexpr int TR = kPdRows, RL = kPdRL;
   extern __shared__ __align__(128) unsigned char smem[];
   const Panel64Smem L(NW, NS);
@@ -254,10 +259,15 @@ __global__ void __launch_bounds__(kPdMaxThreads, 1)
   uint32_t* freed = full + NS;                                  // releases, NW per pass
   volatile uint32_t* bad = full + 2 * NS;                       // Inf or NaN met in the block
   const int lane = threadIdx.x & 31;
-  // panels dealt to warps from a start that moves with the CTA: their work
-  // differs, warp w sits on sub-partition w mod 4 in every CTA, and an SM's
-  // first CTAs are a device's SM count apart
-  const int q = static_cast<int>((threadIdx.x / 32 + blockIdx.x + blockIdx.x / 152u) % static_cast<unsigned>(NW));
+  // Panels differ in work and warp w sits on sub-partition w mod 4 in every CTA:
+  // order deals them evenly (choose_panel); with one warp a sub-partition the
+  // start moves with the CTA instead, an SM's first CTAs being a device's SM
+  // count apart.  (The moving start at every n: Step 1 of 2,000,000 x 50
+  // 10.06 ms, 7.69 dealt evenly; x 40 5.76 and 4.79; 4,000,000 x 64 21.8 and
+  // 20.9; 1,000,000 x 72 7.79 and 6.60.)
+  const unsigned w = threadIdx.x / 32;
+  const int q = NW > 4 ? static_cast<int>((order >> (4 * w)) & 15u)
+                       : static_cast<int>((w + blockIdx.x + blockIdx.x / 152u) % static_cast<unsigned>(NW));
   const int g = lane >> 2, t4 = lane & 3;
   const int64_t row0 = static_cast<int64_t>(blockIdx.x) * b;
   const int rows = static_cast<int>(m - row0 < b ? m - row0 : b);

@@ -139,6 +139,18 @@ bool choose_cfg(int kind, int n, KernelCfg* out, int64_t want_b, int policy, int
 PanelCfg choose_panel(int n) {
   PanelCfg c;
   c.NW = (n + kPdCols - 1) / kPdCols;
+  // panel p takes p block reflectors and its own columns: weight p + 1, the
+  // heaviest first to the sub-partition (warp w runs on w mod 4) with the least
+  // work that has a warp left
+  int load[4] = {0, 0, 0, 0}, used[4] = {0, 0, 0, 0};
+  for (int p = c.NW - 1; p >= 0; --p) {
+    int s = -1;
+    for (int i = 0; i < 4; ++i)
+      if (4 * used[i] + i < c.NW && (s < 0 || load[i] < load[s])) s = i;
+    c.order |= static_cast<uint64_t>(p) << (4 * (4 * used[s] + s));
+    load[s] += p + 1;
+    ++used[s];
+  }
   const int entries = c.NW - 1;  // published panels per tile
   for (c.ctas = kPdMaxThreads / 32 / c.NW; c.ctas >= 1; --c.ctas) {
     const size_t lim = c.ctas == 1 ? kSmemMax : kSmemPerSM / c.ctas - 1024;

@@ -57,6 +57,7 @@ bool choose_cfg(int kind, int n, KernelCfg* out, int64_t want_b = 0, int policy 
 struct PanelCfg {
   int NW = 0, NS = 0, ctas = 1;
   size_t smem = 0;
+  uint64_t order = 0;  // the panel of warp w: bits 4 w .. 4 w + 3
 };
 PanelCfg choose_panel(int n);
 
