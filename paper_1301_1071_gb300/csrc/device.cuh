@@ -123,6 +123,30 @@ __device__ __forceinline__ void bulk_g2s(void* dst_smem, const void* src_gmem, u
       : "memory");
 }
 
+// binary64 <-> binary32, the same results as the conversions, which take 64 clocks
+// a warp on the sub-partition's binary64 unit (idle lanes included): integer
+// operations for zeros and for normal numbers of binary32's range.  4,000,000 x 64
+// binary32: Step 1, which writes T's Gram, 5.24 -> 5.17 ms, the W chain and
+// product of Step 3 0.716 -> 0.680, native Step 3 1.58 -> 1.51.  (Not in
+// k_form_q_tcw, x 100 3.37 -> 3.43 ms, nor in k_build_t, where it changed nothing.)
+__device__ __forceinline__ float f32_of(double x) {
+  const uint32_t hi = static_cast<uint32_t>(__double2hiint(x)), lo = static_cast<uint32_t>(__double2loint(x));
+  const uint32_t mag = hi & 0x7fffffffu;
+  if (mag - 0x38100000u < 0x0fe00000u) {  // 2^-126 <= |x| < 2^128: to nearest, ties to even
+    const uint32_t f = ((mag - 0x38000000u) << 3) | (lo >> 29);
+    return __uint_as_float((hi & 0x80000000u) | (f + (((lo & 0x1fffffffu) + 0x0fffffffu + (f & 1u)) >> 29)));
+  }
+  if ((mag | lo) == 0) return __uint_as_float(hi);
+  return static_cast<float>(x);
+}
+__device__ __forceinline__ double f64_of(float x) {
+  const uint32_t b = __float_as_uint(x), mag = b & 0x7fffffffu;
+  if (mag - 0x00800000u < 0x7f000000u)  // normal
+    return __hiloint2double(static_cast<int>((b & 0x80000000u) | ((mag >> 3) + 0x38000000u)), static_cast<int>(b << 29));
+  if (mag == 0) return __hiloint2double(static_cast<int>(b), 0);
+  return static_cast<double>(x);
+}
+
 // shared -> global bulk copy (bulk-group completion)
 __device__ __forceinline__ void bulk_s2g(void* dst_gmem, const void* src_smem, uint32_t bytes) {
   asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst_gmem),

@@ -28,8 +28,8 @@
 //
 // Measured: Step 1 of 4,000,000 x 64 65.2 -> 20.9 ms plus 3.2 for T's Gram (its
 // bytes 0.6; 2 m n^2 binary64 flops would take 27), 3,000,000 x 32 10.96 -> 5.68.
-// Bound by the chain of panels a tile runs through: the binary64 unit is 44 to
-// 57 % busy with conversions, the columns and T_p^T.
+// Bound by the chain of panels a tile runs through: the binary64 unit is 42 %
+// busy with conversions, the columns and T_p^T.
 #pragma once
 
 #include <cstdint>

@@ -259,7 +259,8 @@ int make_plan(int64_t m, int64_t n, int esz, int64_t block_rows, int fanout, Pla
   // rows, tile -> panels: n = 8 0.81 -> 0.72 ms, 10 0.87 -> 1.54, 12 1.75 -> 1.67,
   // 16 3.03 -> 1.88, 17 2.87 -> 3.40, 20 3.19 -> 3.74, 24 5.43 -> 3.85, 25 5.41 ->
   // 5.28 (with more, shorter tiles for the T factors and Step 3 to take), 28
-  // 7.26 -> 5.88, 32 10.96 -> 5.70, 48 30.9 -> 11.5
+  // 7.26 -> 5.88, 32 10.96 -> 5.70, 48 30.9 -> 11.5 (2,000,000 rows 7.64, and 6.31
+  // since the panels are dealt evenly)
   P.panel = kind0 == kKindF64 && n >= kSplitMinN &&
             !(n <= 25 && (n + 4) / 5 * 5 + 3 < (n + kPdCols - 1) / kPdCols * kPdCols);
   if (P.panel) P.pq = choose_panel((int)n);

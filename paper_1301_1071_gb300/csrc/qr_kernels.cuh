@@ -130,6 +130,11 @@ __device__ __forceinline__ Reflector<T> make_reflector(T Sj, T alpha) {
   }
   return f;
 }
+template <class V>
+__device__ __forceinline__ double slot_of(V v) {  // a value as a T slot holds it
+  if constexpr (sizeof(V) == 4) return f64_of(v);
+  else return static_cast<double>(v);
+}
 // binary64 <-> binary32 by integer operations (normal numbers in binary32's
 // range; towards zero): a conversion costs a slot of the binary64 unit.
 __device__ __forceinline__ float float_of(double x) {
@@ -854,9 +859,9 @@ __global__ void __launch_bounds__(MAXT, 1) k_local_qr(const S* __restrict__ A, i
           // row i by a warp, its entries kk >= i by the lanes (no division)
           for (int i = warp; i < n; i += NW)
             for (int kk = i + lane; kk < n; kk += 32)
-              Tout[i * n + kk] = static_cast<double>(kk > i ? gram[i * n + kk] : taus[i]);
+              Tout[i * n + kk] = slot_of(kk > i ? gram[i * n + kk] : taus[i]);
         } else {
-          for (int i = tid; i < n; i += NT) Tout[i * n + i] = static_cast<double>(taus[i]);
+          for (int i = tid; i < n; i += NT) Tout[i * n + i] = slot_of(taus[i]);
         }
       }
       __syncthreads();

@@ -8,7 +8,7 @@
 // the FMA rate at n = 64.  Row tiles arrive by cp.async one tile ahead, in rows
 // padded to ld = 4 mod 8 floats (conflict-free 16-byte reads of adjacent rows).
 // 4,000,000 x 64: out = X M1 + Y M2 4.27 -> 1.80 ms (bound by the FMA pipe:
-// 32.8 G FMA at 19,456 a clock 0.85 ms, the 3.07 GB 0.46), Step 3 5.04 -> 1.58 ms.
+// 32.8 G FMA at 19,456 a clock 0.85 ms, the 3.07 GB 0.46), Step 3 5.04 -> 1.51 ms.
 #pragma once
 
 #include <cstdint>
@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(208, 2)
     }
     for (int i = threadIdx.x; i < n * n; i += blockDim.x) {
       const int r = i / n, k = i - r * n;
-      tt[r * ld + k] = k >= r ? static_cast<float>(Tb[i]) : 0.0f;
+      tt[r * ld + k] = k >= r ? f32_of(Tb[i]) : 0.0f;
     }
     __syncthreads();
     r32_zero(acc);

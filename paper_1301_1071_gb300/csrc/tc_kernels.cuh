@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(kWcThreads, 3)
       const int idx = tid + e * kWcThreads;
       if (idx < nn) {
         const int kk = idx / n, i = idx - kk * n;
-        ts[i * np + kk] = i >= kk ? static_cast<float>(tp[e]) : 0.0f;
+        ts[i * np + kk] = i >= kk ? f32_of(tp[e]) : 0.0f;
       }
     }
     if (t > 0) fetch_t(t - 1);
