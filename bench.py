@@ -121,8 +121,8 @@ def load_peaks():
 # traffic bench.py reports from a committed ncu capture.
 KERNEL_SOURCES = ["qr_kernels.cuh", "device.cuh", "df64.cuh", "layout.cuh", "kern_inst.cuh", "kern_f64.cu",
                   "kern_df64.cu", "kern_f32.cu", "kern_r_f64.cu", "tiles_f64.h", "tiles_f32.h", "plan.cu", "plan.h",
-                  "split.cuh", "split_kernels.cuh", "rows32.cuh", "kern_rows32.cu", "kern_split.cu", "panel64.cuh", "kern_panel64.cu", "tcgen05.cuh",
-                  "chunks.cuh"]
+                  "split.cuh", "split_kernels.cuh", "kern_split.cu", "rows32.cuh", "kern_rows32.cu", "panel64.cuh",
+                  "kern_panel64.cu", "tcgen05.cuh", "chunks.cuh"]
 
 
 def kernel_source_hash() -> str:
