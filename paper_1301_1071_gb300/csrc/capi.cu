@@ -20,14 +20,14 @@ cudaError_t launch_local_qr_f64(const KernelCfg&, const void*, int64_t, int, int
 cudaError_t launch_local_qr_f32(const KernelCfg&, const void*, int64_t, int, int64_t, int64_t, int, int64_t, void*, double*,
                                 double*, int32_t*, cudaStream_t);
 cudaError_t launch_form_q_f64(const KernelCfg&, const void*, int64_t, int, int64_t, int, int64_t, int, int64_t, const double*,
-                              const double*, int64_t, void*, int32_t*, cudaStream_t);
+                              const double*, int64_t, bool, void*, int32_t*, cudaStream_t);
 cudaError_t launch_form_q_f32(const KernelCfg&, const void*, int64_t, int, int64_t, int, int64_t, int, int64_t, const double*,
-                              const double*, int64_t, void*, int32_t*, cudaStream_t);
+                              const double*, int64_t, bool, void*, int32_t*, cudaStream_t);
 
 cudaError_t launch_local_qr_df64(const KernelCfg&, const void*, int64_t, int, int64_t, int64_t, int, int64_t, void*, double*,
                                  double*, int32_t*, cudaStream_t);
 cudaError_t launch_form_q_df64(const KernelCfg&, const void*, int64_t, int, int64_t, int, int64_t, int, int64_t, const double*,
-                               const double*, int64_t, void*, int32_t*, cudaStream_t);
+                               const double*, int64_t, bool, void*, int32_t*, cudaStream_t);
 cudaError_t launch_local_r_f64(const KernelCfg&, const void*, int64_t, int, int64_t, int64_t, int, int64_t, double*,
                                int32_t*, cudaStream_t);
 cudaError_t launch_local_r_f32(const KernelCfg&, const void*, int64_t, int, int64_t, int64_t, int, int64_t, double*,
@@ -108,15 +108,15 @@ cudaError_t launch_step1(const Plan& P, const void* A, int64_t m, int64_t b, int
 }
 
 cudaError_t launch_form_q(const KernelCfg& k, const void* Y, int64_t m, int n, int64_t b, int B, int64_t bt, int kt,
-                          int64_t p, const double* T, const double* C, int64_t cblocks, void* Q, int32_t* status,
-                          cudaStream_t st) {
+                          int64_t p, const double* T, const double* C, int64_t cblocks, bool comp, void* Q,
+                          int32_t* status, cudaStream_t st) {
   switch (k.kind) {
-    case kKindF64: return launch_form_q_f64(k, Y, m, n, b, B, bt, kt, p, T, C, cblocks, Q, status, st);
+    case kKindF64: return launch_form_q_f64(k, Y, m, n, b, B, bt, kt, p, T, C, cblocks, comp, Q, status, st);
     case kKindF32:
       if (step3_rows32(n) && Y == Q)
         return launch_form_q_f32_tiles(static_cast<float*>(Q), m, n, b, B, bt, kt, p, T, C, cblocks, st);
-      return launch_form_q_f32(k, Y, m, n, b, B, bt, kt, p, T, C, cblocks, Q, status, st);
-    case kKindDF64: return launch_form_q_df64(k, Y, m, n, b, B, bt, kt, p, T, C, cblocks, Q, status, st);
+      return launch_form_q_f32(k, Y, m, n, b, B, bt, kt, p, T, C, cblocks, comp, Q, status, st);
+    case kKindDF64: return launch_form_q_df64(k, Y, m, n, b, B, bt, kt, p, T, C, cblocks, comp, Q, status, st);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -351,10 +351,10 @@ tsqr_status run_direct(const Plan& P, const void* A, void* Q, double* R, int64_t
   const int64_t cb0 = (L == 1) ? 1 : l0.p;
   const cudaError_t e3 =
       P.split3 ? launch_form_q_split(static_cast<double*>(Q), P.m, n, l0.b, P.B0, l0.bt, l0.kt, l0.p, T(0), C0, cb0,
-                                     status, st)
+                                     P.panel, status, st)
       : P.tc3 ? launch_form_q_tc(static_cast<float*>(Q), P.m, n, l0.b, P.B0, l0.bt, l0.kt, l0.p, T(0), C0, cb0,
                                  status, st)
-              : launch_form_q(P.cfg0, Q, P.m, n, l0.b, P.B0, l0.bt, l0.kt, l0.p, T(0), C0, cb0, Q, status, st);
+              : launch_form_q(P.cfg0, Q, P.m, n, l0.b, P.B0, l0.bt, l0.kt, l0.p, T(0), C0, cb0, P.panel, Q, status, st);
   if (e3 != cudaSuccess) return TSQR_ERR_CUDA;
   return mark(o, 3, st);
 }
@@ -526,11 +526,11 @@ tsqr_status run_direct_host(const Plan& P, int chunks, const char* A, char* Qh, 
     const int64_t cb = (L == 1) ? 1 : pcnt;
     char* Y = dbuf + r0 * row_bytes;
     TSQR_CUDA(P.split3 ? launch_form_q_split(reinterpret_cast<double*>(Y), rows, n, l0.b, P.B0, l0.bt, l0.kt,
-                                             pcnt, T0 + b0 * l0.kt * nn, Cc, cb, status, st)
+                                             pcnt, T0 + b0 * l0.kt * nn, Cc, cb, P.panel, status, st)
               : P.tc3 ? launch_form_q_tc(reinterpret_cast<float*>(Y), rows, n, l0.b, P.B0, l0.bt, l0.kt, pcnt,
                                          T0 + b0 * l0.kt * nn, Cc, cb, status, st)
-                      : launch_form_q(P.cfg0, Y, rows, n, l0.b, P.B0, l0.bt, l0.kt, pcnt, T0 + b0 * l0.kt * nn, Cc, cb, Y,
-                                      status, st));
+                      : launch_form_q(P.cfg0, Y, rows, n, l0.b, P.B0, l0.bt, l0.kt, pcnt, T0 + b0 * l0.kt * nn, Cc, cb, P.panel,
+                                      Y, status, st));
     TSQR_CUDA(cudaEventRecord(ev_q[c], st));
     TSQR_CUDA(cudaStreamWaitEvent(cst, ev_q[c], 0));
     TSQR_CUDA(cudaMemcpyAsync(Qh + r0 * row_bytes, Y, rows * row_bytes, cudaMemcpyDeviceToHost, cst));

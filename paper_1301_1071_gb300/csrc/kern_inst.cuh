@@ -29,14 +29,14 @@ static cudaError_t local_qr_R(const KernelCfg& k, const TSQR_S* A, int64_t m, in
 
 template <int R, int MAXT, int NPC>
 static cudaError_t form_q_R(const KernelCfg& k, const TSQR_S* Y, int64_t m, int n, int64_t b, int B, int64_t bt, int kt,
-                            int64_t p, const double* T, const double* C, int64_t cblocks, TSQR_S* Q,
+                            int64_t p, const double* T, const double* C, int64_t cblocks, bool comp, TSQR_S* Q,
                             int32_t* status, cudaStream_t st) {
   if (k.NT > MAXT) return cudaErrorInvalidConfiguration;
   auto fn = k_form_q<TSQR_S, TSQR_T, NPC, R, MAXT>;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem_fq);
   if (e != cudaSuccess) return e;
   fn<<<(unsigned)p, k.NT, k.smem_fq, st>>>(Y, m, n, (int)b, B, (int)bt, kt, k.fq_rows, k.CS, k.NRG, k.skew, T, C,
-                                           cblocks, Q, status);
+                                           cblocks, comp, Q, status);
   return cudaGetLastError();
 }
 
@@ -57,18 +57,18 @@ cudaError_t TSQR_LOCAL_QR_NAME(const KernelCfg& k, const void* A, int64_t m, int
 }
 
 cudaError_t TSQR_FORM_Q_NAME(const KernelCfg& k, const void* Y, int64_t m, int n, int64_t b, int B, int64_t bt, int kt,
-                             int64_t p, const double* T, const double* C, int64_t cblocks, void* Q,
+                             int64_t p, const double* T, const double* C, int64_t cblocks, bool comp, void* Q,
                              int32_t* status, cudaStream_t st) {
   const TSQR_S* y = static_cast<const TSQR_S*>(Y);
   TSQR_S* q = static_cast<TSQR_S*>(Q);
   switch (k.tile) {
-    case 0: return form_q_R<TSQR_R0, TSQR_T0, kNpc>(k, y, m, n, b, B, bt, kt, p, T, C, cblocks, q, status, st);
-    case 1: return form_q_R<TSQR_R1, TSQR_T1, kNpc>(k, y, m, n, b, B, bt, kt, p, T, C, cblocks, q, status, st);
-    case 2: return form_q_R<TSQR_R2, TSQR_T2, kNpc>(k, y, m, n, b, B, bt, kt, p, T, C, cblocks, q, status, st);
-    case 3: return form_q_R<TSQR_R3, TSQR_T3, kNpc>(k, y, m, n, b, B, bt, kt, p, T, C, cblocks, q, status, st);
-    case 4: return form_q_R<TSQR_R4, TSQR_T4, kNpc>(k, y, m, n, b, B, bt, kt, p, T, C, cblocks, q, status, st);
-    case 5: return form_q_R<TSQR_R5, TSQR_T5, TSQR_N5>(k, y, m, n, b, B, bt, kt, p, T, C, cblocks, q, status, st);
-    case 6: return form_q_R<TSQR_R6, TSQR_T6, TSQR_N6>(k, y, m, n, b, B, bt, kt, p, T, C, cblocks, q, status, st);
+    case 0: return form_q_R<TSQR_R0, TSQR_T0, kNpc>(k, y, m, n, b, B, bt, kt, p, T, C, cblocks, comp, q, status, st);
+    case 1: return form_q_R<TSQR_R1, TSQR_T1, kNpc>(k, y, m, n, b, B, bt, kt, p, T, C, cblocks, comp, q, status, st);
+    case 2: return form_q_R<TSQR_R2, TSQR_T2, kNpc>(k, y, m, n, b, B, bt, kt, p, T, C, cblocks, comp, q, status, st);
+    case 3: return form_q_R<TSQR_R3, TSQR_T3, kNpc>(k, y, m, n, b, B, bt, kt, p, T, C, cblocks, comp, q, status, st);
+    case 4: return form_q_R<TSQR_R4, TSQR_T4, kNpc>(k, y, m, n, b, B, bt, kt, p, T, C, cblocks, comp, q, status, st);
+    case 5: return form_q_R<TSQR_R5, TSQR_T5, TSQR_N5>(k, y, m, n, b, B, bt, kt, p, T, C, cblocks, comp, q, status, st);
+    case 6: return form_q_R<TSQR_R6, TSQR_T6, TSQR_N6>(k, y, m, n, b, B, bt, kt, p, T, C, cblocks, comp, q, status, st);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -26,7 +26,8 @@ cudaError_t launch_rowmul_split(const double* X, const double* M, const double* 
 }
 
 cudaError_t launch_form_q_split(double* Y, int64_t m, int n, int64_t b, int B, int64_t bt, int kt, int64_t p,
-                                const double* T, const double* C, int64_t cblocks, int32_t* status, cudaStream_t st) {
+                                const double* T, const double* C, int64_t cblocks, bool comp, int32_t* status,
+                                cudaStream_t st) {
   if (n < 1 || n > kRsMaxN) return cudaErrorInvalidValue;
   const size_t smem = FormQSplitSmem(n).total;
   const int KC = split_kc(n);
@@ -37,7 +38,7 @@ cudaError_t launch_form_q_split(double* Y, int64_t m, int n, int64_t b, int B, i
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   fn<<<static_cast<unsigned>(p), kRsThreads, smem, st>>>(Y, m, n, static_cast<int>(b), B, static_cast<int>(bt), kt, T,
-                                                         C, cblocks, status);
+                                                         C, cblocks, comp, status);
   return cudaGetLastError();
 }
 

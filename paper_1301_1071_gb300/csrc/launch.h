@@ -19,9 +19,10 @@ cudaError_t launch_local_qr(const KernelCfg& k, const void* A, int64_t m, int n,
 // Y, R and tau, or (Y == NULL) R only.
 cudaError_t launch_panel_qr_f64(const PanelCfg& k, const void* A, int64_t m, int n, int64_t b, int kt, int64_t p,
                                 void* Y, double* Rst, double* Tst, int32_t* status, cudaStream_t st);
-// Step 3: p CTAs (B, bt: the tile geometry of Step 1).
+// Step 3: p CTAs (B, bt: the tile geometry of Step 1; comp: the T slots hold 2 -
+// tau, comp_at).
 cudaError_t launch_form_q(const KernelCfg& k, const void* Y, int64_t m, int n, int64_t b, int B, int64_t bt, int kt,
-                          int64_t p, const double* T, const double* C, int64_t cblocks, void* Q,
+                          int64_t p, const double* T, const double* C, int64_t cblocks, bool comp, void* Q,
                           int32_t* status, cudaStream_t st);
 
 // Step-2 up pass of one tree level (binary64): node b = f stacked
@@ -75,9 +76,10 @@ constexpr bool rows_by_digits(int64_t n) { return n >= kSplitMinN && n <= kRowSp
 cudaError_t launch_rowmul_split(const double* X, const double* M, const double* colsrc, const int* colexp, int64_t m,
                                 int n, bool add, double* out, int32_t* status, cudaStream_t st);
 // Step 3 for binary64 data, n <= kRowSplitMaxN; the block and tile geometry of
-// Step 1, Q over Y.
+// Step 1, Q over Y.  comp: the T slots hold 2 - tau (comp_at).
 cudaError_t launch_form_q_split(double* Y, int64_t m, int n, int64_t b, int B, int64_t bt, int kt, int64_t p,
-                                const double* T, const double* C, int64_t cblocks, int32_t* status, cudaStream_t st);
+                                const double* T, const double* C, int64_t cblocks, bool comp, int32_t* status,
+                                cudaStream_t st);
 // Partial Grams X^T Y into at most max_parts n x n partials (*parts written);
 // colexp (or NULL): n ints, zeroed by the caller, receiving the largest binary
 // exponents of X's columns.

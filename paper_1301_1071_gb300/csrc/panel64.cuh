@@ -61,7 +61,7 @@ struct Panel64Smem {
     slots = o; o = align_up(o + NS * kPdSlotBytes, 128);
     tiles = o; o += NW * kPdTileBytes;
     r = o; o += static_cast<size_t>(kPdCols * kPdCols) * 8 * NW * (NW + 1) / 2;  // warp q: 8 (q + 1) rows
-    wbuf = o; o += static_cast<size_t>(NW) * 3 * kPdCols * 8;                    // two buffers of sums, pivot row
+    wbuf = o; o += static_cast<size_t>(NW) * 5 * kPdCols * 8;  // two buffers of sums, pivot row, tau, 2 - tau
     total = align_up(o, 16);
   }
 };
@@ -152,10 +152,11 @@ __device__ __forceinline__ long long fixed_of(double x, int sc) {
 }
 
 // One column of the panel factorisation (rows lane + 32 i in a[i]).
-// rbuf: the pivot row (tile 0) is exchanged there; sbuf: the sums.
+// rbuf: the pivot row (tile 0) is exchanged there, then the panel's tau and 2 -
+// tau; sbuf: the sums.
 template <int J>
 __device__ __forceinline__ void panel64_column(double (&a)[kPdRL][kPdCols], double* Rq, double* sbuf, double* rbuf,
-                                               int j0, int nb, bool first, int lane, double& tau_j) {
+                                               int j0, int nb, bool first, int lane) {
   const int r = j0 + J;
   const double* prow = Rq + r * kPdCols;
   if (first) {
@@ -192,16 +193,24 @@ __device__ __forceinline__ void panel64_column(double (&a)[kPdRL][kPdCols], doub
   __syncwarp();
   const double alpha = prow[J], sj = dst[J];
   const Reflector<double> f = make_reflector64(fma(alpha, alpha, sj), alpha);
-  tau_j = f.tau;
+  // 2 - tau = s_J / (root (|alpha| + root)), with a relative error of its own:
+  // taken from the rounded tau it errs by tau's rounding, which a block's every
+  // tile adds to Q
+  const double ps = sj * f.scal;
+  if (lane == 0) {
+    rbuf[kPdCols + J] = f.tau;
+    rbuf[2 * kPdCols + J] = f.ident ? 2.0 : -ps * f.ib;
+  }
   // lane c: column c's row of R and its coefficient of x.  r' = (alpha r + s) /
-  // beta as -r + (s + (alpha + beta) r) / beta with alpha + beta = -s_J /
-  // (alpha - beta): in a block's later tiles alpha is close to -beta, so the
-  // correction is small and the running R takes one rounding a tile
+  // beta, from tile 1 on as -r + (s + (alpha + beta) r) / beta with alpha + beta
+  // = -s_J / (alpha - beta): there alpha is close to -beta, so the correction is
+  // small and the running R takes one rounding a tile (in tile 0 alpha is one
+  // entry, and that form would cancel)
   double dl = 0.0, rn = 0.0;
   const bool trail = lane > J && lane < nb;
   if (trail) {
     const double rc = prow[lane];
-    rn = f.ident ? rc : fma(fma(-sj * f.scal, rc, dst[lane]), f.ib, -rc);
+    rn = f.ident ? rc : first ? fma(alpha, rc, dst[lane]) * f.ib : fma(fma(-ps, rc, dst[lane]), f.ib, -rc);
     dl = (rn - rc) * f.scal;
   }
   __syncwarp();  // the pivot row has been read
@@ -230,12 +239,11 @@ __device__ __forceinline__ void panel64_column(double (&a)[kPdRL][kPdCols], doub
 // Columns J .. nb - 1 (the padding columns of a last panel are zero: they give
 // zero vectors and tau = 0).
 template <int J>
-__device__ __forceinline__ void panel64_factor(double (&a)[kPdRL][kPdCols], double (&tau)[kPdCols], double* Rq,
-                                               double* sbuf, double* rbuf, int j0, int nb, bool first, int lane) {
+__device__ __forceinline__ void panel64_factor(double (&a)[kPdRL][kPdCols], double* Rq, double* sbuf, double* rbuf,
+                                               int j0, int nb, bool first, int lane) {
   if constexpr (J < kPdCols) {
-    tau[J] = 0.0;
-    if (J < nb) panel64_column<J>(a, Rq, sbuf, rbuf, j0, nb, first, lane, tau[J]);
-    panel64_factor<J + 1>(a, tau, Rq, sbuf, rbuf, j0, nb, first, lane);
+    if (J < nb) panel64_column<J>(a, Rq, sbuf, rbuf, j0, nb, first, lane);
+    panel64_factor<J + 1>(a, Rq, sbuf, rbuf, j0, nb, first, lane);
   }
 }
 
@@ -280,7 +288,7 @@ __global__ void __launch_bounds__(kPdMaxThreads, 1)
 
   const int j0 = kPdCols * q, nb = n - j0 < kPdCols ? n - j0 : kPdCols;
   double* Rq = reinterpret_cast<double*>(smem + L.r) + kPdCols * kPdCols * q * (q + 1) / 2;
-  double* sbuf = reinterpret_cast<double*>(smem + L.wbuf) + static_cast<size_t>(q) * 3 * kPdCols;
+  double* sbuf = reinterpret_cast<double*>(smem + L.wbuf) + static_cast<size_t>(q) * 5 * kPdCols;
   double* rbuf = sbuf + 2 * kPdCols;
   long long* X = reinterpret_cast<long long*>(smem + L.tiles + static_cast<size_t>(q) * kPdTileBytes);
   double* Xd = reinterpret_cast<double*>(X);
@@ -508,8 +516,7 @@ __global__ void __launch_bounds__(kPdMaxThreads, 1)
     for (int i = 0; i < RL; ++i)
 #pragma unroll
       for (int c = 0; c < kPdCols; ++c) a[i][c] = Xd[tile_at(lane + 32 * i, c)];
-    double tau[kPdCols];
-    panel64_factor<0>(a, tau, Rq, sbuf, rbuf, j0, nb, first, lane);
+    panel64_factor<0>(a, Rq, sbuf, rbuf, j0, nb, first, lane);
     // ---- V through the tile: digits (62-bit fixed point per column) and Y
 #pragma unroll
     for (int i = 0; i < RL; ++i)
@@ -604,12 +611,12 @@ __global__ void __launch_bounds__(kPdMaxThreads, 1)
         double s = 0.0;
 #pragma unroll
         for (int l = 0; l < J; ++l) s = fma(tr[l], T[l * kPdCols + J], s);
-        tr[J] = lane < J ? -tau[J] * s : (lane == J ? tau[J] : 0.0);
+        tr[J] = lane < J ? -rbuf[kPdCols + J] * s : (lane == J ? rbuf[kPdCols + J] : 0.0);
       }
       __syncwarp();
       if (lane < kPdCols) {
 #pragma unroll
-        for (int c = 0; c < kPdCols; ++c) T[lane * kPdCols + c] = (lane == c ? 2.0 : 0.0) - tr[c];  // E = 2 I - T
+        for (int c = 0; c < kPdCols; ++c) T[lane * kPdCols + c] = lane == c ? rbuf[2 * kPdCols + c] : -tr[c];  // E = 2 I - T
       }
       __syncwarp();
       if (lane == 0) {
@@ -629,7 +636,10 @@ __global__ void __launch_bounds__(kPdMaxThreads, 1)
       double* Tg = Tst + (static_cast<int64_t>(blockIdx.x) * kt + t) * n * n;
 #pragma unroll
       for (int c = 0; c < kPdCols; ++c)
-        if (lane == c && c < nb) Tg[static_cast<int64_t>(j0 + c) * (n + 1)] = tau[c];
+        if (lane == c && c < nb) {
+          Tg[static_cast<int64_t>(j0 + c) * (n + 1)] = rbuf[kPdCols + c];
+          Tg[comp_at(j0 + c, n)] = rbuf[2 * kPdCols + c];
+        }
       __syncwarp();
     }
   }

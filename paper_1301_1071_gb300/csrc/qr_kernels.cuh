@@ -933,6 +933,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_local_qr(const S* __restrict__ A, i
 //   Yg  : m x n (storage S), as written by Step 1 (tiles of B, then bt rows).
 //   Tg  : kt slots of n x n binary64 per block (T of each tile, upper part).
 //   Cg  : cblocks blocks of n x n binary64 (cblocks == 1: one C for all).
+//   comp: the T slots hold 2 - tau (comp_at; binary64 data by panels).
 //   Qg  : output m x n (storage S); may alias Yg.
 // The n x n operands stream through the stage in row chunks; each thread
 // keeps its (at most kMaxE) entries of an n x NPAD product in registers.
@@ -947,8 +948,8 @@ constexpr int max_entries() { return (NPC * 100 + 31) / 32; }  // n <= 100
 template <class S, class T, int NPC, int R, int MAXT>
 __global__ void __launch_bounds__(MAXT, 1) k_form_q(const S* Yg, int64_t m, int n, int b, int B, int bt, int kt, int srows,
                                                      int CS, int NRG, int skew, const double* __restrict__ Tg,
-                                                     const double* __restrict__ Cg, int64_t cblocks, S* Qg,
-                                                     int32_t* status) {
+                                                     const double* __restrict__ Cg, int64_t cblocks, bool comp,
+                                                     S* Qg, int32_t* status) {
   extern __shared__ __align__(128) unsigned char smem[];
   const int NT = blockDim.x;
   const int NPAD = NPC * CS;
@@ -1035,7 +1036,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_form_q(const S* Yg, int64_t m, int 
       for (int e = 0; e < kMaxE; ++e) {
         const int idx = tid + e * NT, kk = idx / NPAD, c = idx % NPAD;
         if (idx < NE && c < n && kk >= k0 && kk < k1)
-          for (int i = kk; i < n; ++i) w[e] = fma(tm[(kk - k0) * n + i], src[i * NPAD + c], w[e]);
+          for (int i = kk + (comp ? 1 : 0); i < n; ++i) w[e] = fma(tm[(kk - k0) * n + i], src[i * NPAD + c], w[e]);
       }
       __syncthreads();
     }
@@ -1043,8 +1044,16 @@ __global__ void __launch_bounds__(MAXT, 1) k_form_q(const S* Yg, int64_t m, int 
     for (int e = 0; e < kMaxE; ++e) {
       const int idx = tid + e * NT;
       if (idx < NE) {
+        if (std::is_same<T, double>::value && comp) {
+          // the strict triangle's sum so far; X - W = -X + ((2 - tau) X - sum)
+          const int kk = idx / NPAD;
+          const T x = src[idx];
+          if (t > 0) Xm[idx] = fma(T(Tb[comp_at(kk, n)]), x, -w[e]) - x;
+          w[e] = fma(T(Tb[kk * (n + 1)]), x, w[e]);
+        } else if (t > 0) {
+          Xm[idx] = Xm[idx] - w[e];  // coefficient of tile t-1
+        }
         Wm[idx] = w[e];
-        if (t > 0) Xm[idx] = Xm[idx] - w[e];  // coefficient of tile t-1
       }
     }
     __syncthreads();

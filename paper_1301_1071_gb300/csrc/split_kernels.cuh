@@ -173,7 +173,7 @@ struct FormQSplitSmem {
 template <int KC>
 __global__ void __launch_bounds__(kRsThreads, KC <= 2 ? 2 : 1)
     k_form_q_split(double* Yg, int64_t m, int n, int b, int B, int bt, int kt, const double* __restrict__ Tg,
-                   const double* __restrict__ Cg, int64_t cblocks, int32_t* status) {
+                   const double* __restrict__ Cg, int64_t cblocks, bool comp, int32_t* status) {
   extern __shared__ __align__(128) unsigned char smem[];
   const FormQSplitSmem L(n);
   uint2* bfrag = reinterpret_cast<uint2*>(smem + L.b);
@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(kRsThreads, KC <= 2 ? 2 : 1)
               wm[r * n + c] = fma(tau, xo, v);
               // the coefficient of tile t - 1, X - W = -X + ((2 - tau) X - v):
               // with tau close to 2 one rounding of X a tile
-              if (!top) xm[r * n + c] = fma(2.0 - tau, xo, -v) - xo;
+              if (!top) xm[r * n + c] = fma(comp ? Tb[comp_at(r, n)] : 2.0 - tau, xo, -v) - xo;
             }
           }
         }

@@ -1,0 +1,40 @@
+"""Accuracy of the binary64 calls against long-double references, beyond the
+bars of the parity tests."""
+import numpy as np
+import pytest
+
+import oracle
+import tsqr_inputs as ti
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+U = 2.0 ** -53  # half an ulp of 1
+
+
+def _T():
+    import paper_1301_1071_gb300 as T
+    return T
+
+
+def _cuda(a):
+    return torch.tensor(np.ascontiguousarray(a), dtype=torch.float64, device="cuda")
+
+
+def _q_error(A, **kw):
+    """||Q - Q_exact||_F / ||Q_exact||_F of the direct call."""
+    Q, _ = _T().direct(_cuda(A), **kw)
+    Qe, _ = oracle.mgs_ld(A)
+    return np.linalg.norm(Q.cpu().numpy() - Qe) / np.linalg.norm(Qe)
+
+
+@pytest.mark.parametrize("n", [8, 16, 48, 64, 72, 100])
+def test_many_tiles_in_a_block(n):
+    """One row block of 64 tiles: what a tile adds is independent of the other
+    tiles' and at most half an ulp of the running R and of the coefficient X
+    (their one rounding a tile), so Q errs by at most sqrt(64) + 1 half ulps,
+    the first tile's own included.  (With 2 - tau taken from the rounded tau, as
+    the tiles' tau come close to 2, it was twice that.)"""
+    tiles = 64
+    errs = [_q_error(ti.gaussian(128 * tiles, n, 900 + s), block_rows=128 * tiles) for s in range(2)]
+    assert max(errs) <= U * (np.sqrt(tiles) + 1), errs
