@@ -152,8 +152,8 @@ __device__ __forceinline__ long long fixed_of(double x, int sc) {
 }
 
 // One column of the panel factorisation (rows lane + 32 i in a[i]).
-// rbuf: the pivot row (tile 0) is exchanged there, then the panel's tau and 2 -
-// tau; sbuf: the sums.
+// rbuf: the pivot row (tile 0) is exchanged there, then the factors of 2 - tau;
+// sbuf: the sums.
 template <int J>
 __device__ __forceinline__ void panel64_column(double (&a)[kPdRL][kPdCols], double* Rq, double* sbuf, double* rbuf,
                                                int j0, int nb, bool first, int lane) {
@@ -193,13 +193,10 @@ __device__ __forceinline__ void panel64_column(double (&a)[kPdRL][kPdCols], doub
   __syncwarp();
   const double alpha = prow[J], sj = dst[J];
   const Reflector<double> f = make_reflector64(fma(alpha, alpha, sj), alpha);
-  // 2 - tau = s_J / (root (|alpha| + root)), with a relative error of its own:
-  // taken from the rounded tau it errs by tau's rounding, which a block's every
-  // tile adds to Q
   const double ps = sj * f.scal;
-  if (lane == 0) {
-    rbuf[kPdCols + J] = f.tau;
-    rbuf[2 * kPdCols + J] = f.ident ? 2.0 : -ps * f.ib;
+  if (lane == 0) {  // the factors of 2 - tau (panel64_tau)
+    rbuf[kPdCols + J] = f.ident ? 2.0 : ps;
+    rbuf[2 * kPdCols + J] = f.ident ? -1.0 : f.ib;
   }
   // lane c: column c's row of R and its coefficient of x.  r' = (alpha r + s) /
   // beta, from tile 1 on as -r + (s + (alpha + beta) r) / beta with alpha + beta
@@ -245,6 +242,20 @@ __device__ __forceinline__ void panel64_factor(double (&a)[kPdRL][kPdCols], doub
     if (J < nb) panel64_column<J>(a, Rq, sbuf, rbuf, j0, nb, first, lane);
     panel64_factor<J + 1>(a, Rq, sbuf, rbuf, j0, nb, first, lane);
   }
+}
+
+// 2 - tau of the panel's columns, lane c for column c (each of the unit's
+// instructions takes a warp 64 clocks, so one for the eight): s_J / (root
+// (|alpha| + root)) with a relative error of its own -- taken from the rounded
+// tau it errs by tau's rounding, which a block's every tile adds to Q.  rbuf then
+// holds tau and 2 - tau.
+__device__ __forceinline__ void panel64_tau(double* rbuf, int lane) {
+  if (lane < kPdCols) {
+    const double eps = -(rbuf[kPdCols + lane] * rbuf[2 * kPdCols + lane]);
+    rbuf[kPdCols + lane] = 2.0 - eps;
+    rbuf[2 * kPdCols + lane] = eps;
+  }
+  __syncwarp();
 }
 
 // ---------------------------------------------------------------------------
@@ -517,6 +528,8 @@ __global__ void __launch_bounds__(kPdMaxThreads, 1)
 #pragma unroll
       for (int c = 0; c < kPdCols; ++c) a[i][c] = Xd[tile_at(lane + 32 * i, c)];
     panel64_factor<0>(a, Rq, sbuf, rbuf, j0, nb, first, lane);
+    __syncwarp();
+    panel64_tau(rbuf, lane);
     // ---- V through the tile: digits (62-bit fixed point per column) and Y
 #pragma unroll
     for (int i = 0; i < RL; ++i)
