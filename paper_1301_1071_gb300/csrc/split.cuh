@@ -4,20 +4,20 @@
 //
 // Splitting (Ozaki, Ogita, Oishi, Rump 2012): a row of the left operand and a
 // column of the right one are fixed-point integers against their largest
-// exponent, |X| <= 2^54 in 7 balanced digits of 8 bits for the rows,
-// X = sum_s d_s 2^(8 (6 - s)), -128 <= d_s <= 127 -- exact in binary16 --, and
-// |X| <= 2^62 in 8 digits for the (few) columns.  The
-// products of a diagonal D = s + t sum to integers of magnitude at most
-// (D + 1) K 2^14, exact in binary32; the diagonals D <= 7 are recombined in
-// 64-bit integers and rounded once to binary64.  What is dropped lies 2^-60
-// (root mean square) below row scale x column scale, and the rows' fixed
-// point rounds at 2^-55 of the row scale (without diagonal 7 it was 2^-52, and
-// Cholesky QR at kappa 1e4 came out 1.8 times further from the exact Q; with 7
-// digits for the columns Step 3 did at 20,000 x 20, 3.8e-16 -> 4.1e-16).
+// exponent, |X| <= 2^62 in 8 balanced digits of 8 bits, X = sum_s d_s 2^(8 (7 -
+// s)), -128 <= d_s <= 127 -- exact in binary16.  The products of a diagonal D =
+// s + t sum to integers of magnitude at most (D + 1) K 2^14, exact in binary32;
+// the diagonals D <= 7 are recombined in 64-bit integers and rounded once to
+// binary64.  What is dropped lies 2^-60 (root mean square) below row scale x
+// column scale; the fixed point itself rounds at 2^-63 of either scale, so the
+// accuracy is normwise: an entry 2^-k of its row's largest keeps 62 - k bits.
+// (Rows of 7 digits, 2^-55, for n > 48 doubled the error of small row entries
+// and put Step 3 of 3,000 x 64 at 5.5e-16, 4.8e-16 with 8; without diagonal 7
+// Cholesky QR at kappa 1e4 came out 1.8 times further from the exact Q.)
 //
 // Why registers: GB300 has 1.9 binary64 FMAs per clock and SM, against 1024
-// binary16 tensor FMAs through mma.sync; 35 digit products per binary64 product
-// leave 16 times the binary64 rate.  What bounds these kernels is the integer
+// binary16 tensor FMAs through mma.sync; 36 digit products per binary64 product
+// leave 15 times the binary64 rate.  What bounds these kernels is the integer
 // unit (64 lanes a clock) that splits and recombines, so digits go straight
 // from the registers that hold an operand's fragment into the product, with no
 // pass through shared memory.
@@ -70,29 +70,6 @@ __device__ __forceinline__ long long split_fixed(double x, int sh) {
   return static_cast<int>(hi) < 0 ? -s : s;
 }
 
-// The 7 balanced digits of a pair of fixed-point values (|X|, |Y| <= 2^54) as
-// binary16 pairs, digit 0 the most significant.  Adding 0x80 to every byte
-// makes the digits unsigned (value + 128); byte 7 becomes 0x64, so that a byte
-// permute forms the binary16 patterns of 1024 + b for the digits in the upper
-// words, and one subtraction leaves b - 128.
-__device__ __forceinline__ void split_digits(long long X, long long Y, uint32_t (&h)[7]) {
-  const unsigned long long bias = 0x6480808080808080ull;
-  const unsigned long long x = static_cast<unsigned long long>(X) + bias, y = static_cast<unsigned long long>(Y) + bias;
-  const uint32_t xl = static_cast<uint32_t>(x), xh = static_cast<uint32_t>(x >> 32);
-  const uint32_t yl = static_cast<uint32_t>(y), yh = static_cast<uint32_t>(y >> 32);
-#pragma unroll
-  for (int s = 0; s < 7; ++s) {
-    const int byte = 6 - s, jb = byte & 3;
-    uint32_t v;
-    if (byte >= 4) {
-      v = __byte_perm(xh, yh, static_cast<uint32_t>(jb | (3 << 4) | ((4 + jb) << 8) | (7 << 12)));
-    } else {
-      v = (__byte_perm(xl, yl, static_cast<uint32_t>(jb | ((4 + jb) << 8))) & 0x00ff00ffu) | 0x64006400u;
-    }
-    asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(h[s]) : "r"(v), "r"(0x64806480u));  // 1024 + 128
-  }
-}
-
 // An accumulator that starts at kSplitMagic holds, in its low bits, the
 // integer sum v, |v| <= 2^22: bits = kSplitMagicBits + v.
 constexpr float kSplitMagic = 12582912.0f;  // 1.5 2^23
@@ -122,17 +99,26 @@ __device__ __forceinline__ double split_to_double(long long P, int s) {
   return __hiloint2double(static_cast<int>((static_cast<uint32_t>(e) << 20) + mh | sign), static_cast<int>(ml));
 }
 
-// sum_D v_D 2^(44 - 8 D), D = 0 .. 7 (the last two rounded): the digit
-// diagonals of a product, in units of 2^60 for a 7-digit operand
-// (|X| <= 2^54) and an 8-digit one (|X| <= 2^62), of 2^68 for two 8-digit ones.  Sums of at
-// most 64 products: |v_D| <= (D + 1) 2^20 keeps every step in 32 bits, and the
-// whole below 2^63.
-__device__ __forceinline__ long long split_combine(const int (&v)[8]) {
-  const int a = v[1] * 256 + v[2];                               // units of 2^28
-  const int b = v[3] * 256 + v[4];                               // of 2^12
-  const int c = v[5] * 16 + ((v[6] * 256 + v[7] + 2048) >> 12);  // of 1
-  return (static_cast<long long>(v[0]) << 44) + (static_cast<long long>(a) << 28) + (static_cast<long long>(b) << 12) +
-         c;
+// sum_D v_D 2^(44 - 8 D), D = 0 .. 7: the digit diagonals of a product of two
+// operands |X| <= 2^62, in units of 2^68, rounded down, and the rest, 0 <= rem <
+// 4096, in units of 2^56.  Sums of at most 64 products: |v_D| <= (D + 1) 2^20
+// keeps every step in 32 bits, and the whole below 2^63.
+__device__ __forceinline__ long long split_combine(const int (&v)[8], int& rem) {
+  const int a = v[1] * 256 + v[2];  // units of 2^28
+  const int b = v[3] * 256 + v[4];  // of 2^12
+  const int l = v[6] * 256 + v[7];  // of 2^-12
+  const int c = v[5] * 16 + (l >> 12);
+  rem = l & 4095;
+  return static_cast<long long>(v[0]) * (1ll << 44) + static_cast<long long>(a) * (1ll << 28) +
+         static_cast<long long>(b) * (1ll << 12) + c;
+}
+// As P 2^e in units of 2^60: rounded to units of 2^68 (e = 8), cut to 2^60 (e =
+// 0) below 2^54 of those, so that P has at least the 53 bits of its rounding
+// wherever the operands give them.
+__device__ __forceinline__ long long split_round(long long o, int rem, int& e) {
+  const bool small = static_cast<uint32_t>(static_cast<int>(o >> 32) + 0x400000) < 0x800000u;
+  e = small ? 0 : 8;
+  return small ? o * 256 + (rem >> 4) : o + (rem >> 11);
 }
 
 // The 8 balanced digits of a pair of fixed-point values (|X|, |Y| <= 2^62).
@@ -225,12 +211,8 @@ __device__ __forceinline__ void split_build_b(F val, int n, int KC, const int* k
 // a[c][s][0..3]: the mma fragment registers of digit s; er[2]: the exponents of
 // the two rows (kExpZero for a zero row; a row with Inf or NaN has 0x7ff or
 // more when kexp is NULL).  load(r, k): the entry of row r (0..15), column k.
-template <int KC>
-constexpr int split_rd() {  // digits of the rows: 8 where the registers hold them (n <= 48)
-  return KC <= 3 ? 8 : 7;
-}
 template <int KC, class F>
-__device__ __forceinline__ void split_rows(F load, int n, const int* kexp, uint32_t (&a)[KC][split_rd<KC>()][4], int (&er)[2],
+__device__ __forceinline__ void split_rows(F load, int n, const int* kexp, uint32_t (&a)[KC][8][4], int (&er)[2],
                                            bool (&bad)[2]) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
 #pragma unroll
@@ -264,14 +246,13 @@ __device__ __forceinline__ void split_rows(F load, int n, const int* kexp, uint3
         int e = static_cast<int>((static_cast<uint32_t>(__double2hiint(x[c][i])) >> 20) & 0x7ffu);
         e = e > 0 ? e : 1;
         if (kexp) e -= kexp[k];
-        f[i] = split_fixed<split_rd<KC>() == 8 ? 62 : 54>(x[c][i], max(em - e, 0));
+        f[i] = split_fixed<62>(x[c][i], max(em - e, 0));
       }
-      constexpr int RD = split_rd<KC>();
-      uint32_t h0[RD], h1[RD];
+      uint32_t h0[8], h1[8];
       split_digits(f[0], f[1], h0);
       split_digits(f[2], f[3], h1);
 #pragma unroll
-      for (int s = 0; s < RD; ++s) {
+      for (int s = 0; s < 8; ++s) {
         a[c][s][h] = h0[s];
         a[c][s][2 + h] = h1[s];
       }
@@ -282,8 +263,8 @@ __device__ __forceinline__ void split_rows(F load, int n, const int* kexp, uint3
 // One column tile: o[0], o[1] = row g at columns 2 t, 2 t + 1 of the tile,
 // o[2], o[3] = row g + 8.  e0 / e1: er + cexp of the entries' columns.
 template <int KC>
-__device__ __forceinline__ void split_product(const uint32_t (&a)[KC][split_rd<KC>()][4], const uint2* bfrag, int lane,
-                                              long long (&o)[4]) {
+__device__ __forceinline__ void split_product(const uint32_t (&a)[KC][8][4], const uint2* bfrag, int lane,
+                                              long long (&o)[4], int (&oe)[4]) {
   // diagonals 4 .. 7 of K > 32 in two halves: |v| stays below 2^22
   constexpr int H = KC > 2 ? 2 : 1;
   float acc[8][4], acc2[H > 1 ? 4 : 1][4];
@@ -303,7 +284,7 @@ __device__ __forceinline__ void split_product(const uint32_t (&a)[KC][split_rd<K
 #pragma unroll
     for (int s = 0; s < 8; ++s) b[s] = bfrag[(c * 8 + s) * 32 + lane];
 #pragma unroll
-    for (int u = 0; u < split_rd<KC>(); ++u)
+    for (int u = 0; u < 8; ++u)
 #pragma unroll
       for (int d = u; d < 8; ++d) {  // digit u of the rows, digit d - u of the columns
         if (H > 1 && d >= 4 && c >= 2)
@@ -321,11 +302,12 @@ __device__ __forceinline__ void split_product(const uint32_t (&a)[KC][split_rd<K
 #pragma unroll
       for (int d = 4; d < 8; ++d) v[d] += split_int(acc2[d - 4][i]);
     }
-    o[i] = split_combine(v);
+    int rem;
+    o[i] = split_combine(v, rem);
+    o[i] = split_round(o[i], rem, oe[i]);
   }
 }
-// value = o 2^(er + cexp - kSplitShift), for either count of row digits: one
-// more byte in the row's fixed point is one more in the unit of the sum
-constexpr int kSplitShift = 2100;
+// value = o 2^(er + cexp + oe - kSplitShift)
+constexpr int kSplitShift = 2108;
 
 }  // namespace tsqr

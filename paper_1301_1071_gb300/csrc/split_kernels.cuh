@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(kRsThreads, KC <= 2 ? 2 : 1)
     __syncwarp();
     const int64_t r0 = tile * kRsRows;
     const int rows = static_cast<int>(m - r0 < kRsRows ? m - r0 : kRsRows);
-    uint32_t a[KC][split_rd<KC>()][4];
+    uint32_t a[KC][8][4];
     int er[2];
     bool bad[2];
     split_rows<KC>([&](int r, int k) { return (r < rows && k < n) ? xs[r * n + k] : 0.0; }, n, scaled ? kx : nullptr,
@@ -112,7 +112,8 @@ __global__ void __launch_bounds__(kRsThreads, KC <= 2 ? 2 : 1)
     issue(tile + stride);
     for (int j = 0; j < NT; ++j) {
       long long o[4];
-      split_product<KC>(a, bfrag + static_cast<size_t>(j) * KC * 8 * 32, lane, o);
+      int oe[4];
+      split_product<KC>(a, bfrag + static_cast<size_t>(j) * KC * 8 * 32, lane, o, oe);
       const int c0 = 8 * j + 2 * t;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
@@ -123,7 +124,7 @@ __global__ void __launch_bounds__(kRsThreads, KC <= 2 ? 2 : 1)
 #pragma unroll
           for (int i = 0; i < 2; ++i) {
             const int ce = cexp[c0 + i];
-            v[i] = split_to_double(o[2 * h + i], er[h] + ce - kSplitShift);
+            v[i] = split_to_double(o[2 * h + i], er[h] + ce + oe[2 * h + i] - kSplitShift);
             if (bad[h] || ce == kExpBad) v[i] = __longlong_as_double(0x7ff8000000000000ll);
           }
           if (c0 + 1 < n && (n & 1) == 0) {
@@ -255,7 +256,7 @@ __global__ void __launch_bounds__(kRsThreads, KC <= 2 ? 2 : 1)
       constexpr int SHARE = NWARP / KC;
       const int rt = warp % KC, part = warp / KC;
       if (part < SHARE) {
-        uint32_t a[KC][split_rd<KC>()][4];
+        uint32_t a[KC][8][4];
         int er[2];
         bool bad[2];
         split_rows<KC>(
@@ -266,12 +267,13 @@ __global__ void __launch_bounds__(kRsThreads, KC <= 2 ? 2 : 1)
             n, nullptr, a, er, bad);
         for (int j = part; j < NT; j += SHARE) {
           long long o[4];
-          split_product<KC>(a, bfrag + static_cast<size_t>(j) * KC * 8 * 32, lane, o);
+          int oe[4];
+          split_product<KC>(a, bfrag + static_cast<size_t>(j) * KC * 8 * 32, lane, o, oe);
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             const int r = 16 * rt + g + 8 * (i >> 1), c = 8 * j + t2 + (i & 1);
             if (r < n && c < n) {
-              double v = split_to_double(o[i], er[i >> 1] + cexp[c] - kSplitShift);
+              double v = split_to_double(o[i], er[i >> 1] + cexp[c] + oe[i] - kSplitShift);
               if (bad[i >> 1] || cexp[c] == kExpBad) v = __longlong_as_double(0x7ff8000000000000ll);
               const double tau = Tb[static_cast<int64_t>(r) * n + r], xo = src[r * n + c];
               wm[r * n + c] = fma(tau, xo, v);
@@ -296,7 +298,7 @@ __global__ void __launch_bounds__(kRsThreads, KC <= 2 ? 2 : 1)
       __syncwarp();
       const int rc = cnt - p0 < kRsRows ? cnt - p0 : kRsRows;
       double* q = Yg + (row0 + tr0 + p0) * n;
-      uint32_t a[KC][split_rd<KC>()][4];
+      uint32_t a[KC][8][4];
       int er[2];
       bool bad[2];
       split_rows<KC>(
@@ -309,7 +311,8 @@ __global__ void __launch_bounds__(kRsThreads, KC <= 2 ? 2 : 1)
       issue();
       for (int j = 0; j < NT; ++j) {
         long long o[4];
-        split_product<KC>(a, bfrag + static_cast<size_t>(j) * KC * 8 * 32, lane, o);
+        int oe[4];
+        split_product<KC>(a, bfrag + static_cast<size_t>(j) * KC * 8 * 32, lane, o, oe);
         const int c0 = 8 * j + t2;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
@@ -319,7 +322,7 @@ __global__ void __launch_bounds__(kRsThreads, KC <= 2 ? 2 : 1)
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
               const int ce = cexp[c0 + i];
-              v[i] = split_to_double(-o[2 * h + i], er[h] + ce - kSplitShift);
+              v[i] = split_to_double(-o[2 * h + i], er[h] + ce + oe[2 * h + i] - kSplitShift);
               if (bad[h] || ce == kExpBad) v[i] = __longlong_as_double(0x7ff8000000000000ll);
               if (top && p0 + r < ntop && c0 + i < n) v[i] += xm[(p0 + r) * n + c0 + i];
             }
@@ -519,7 +522,9 @@ __global__ void __launch_bounds__(MAXT, MINB)
 #pragma unroll
         for (int d = 0; d < 8; ++d) v[d] = split_int(acc[d][i]) + (d >= 4 ? split_int(ac2[d - 4][i]) : 0);
         const int xe = ex[16 * tmi[u] + g + 8 * (i >> 1)], ye = ey[8 * tnj[u] + 2 * t + (i & 1)];
-        double r = split_to_double(split_combine(v), xe + ye - kSplitShift);
+        int rem;
+        const long long o = split_combine(v, rem);
+        double r = split_to_double(o + (rem >> 11), xe + ye + 8 - kSplitShift);
         if (xe >= 0x7ff || ye >= 0x7ff) r = __longlong_as_double(0x7ff8000000000000ll);
         sum[u][i] += r;
       }

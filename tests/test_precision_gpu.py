@@ -38,3 +38,20 @@ def test_many_tiles_in_a_block(n):
     tiles = 64
     errs = [_q_error(ti.gaussian(128 * tiles, n, 900 + s), block_rows=128 * tiles) for s in range(2)]
     assert max(errs) <= U * (np.sqrt(tiles) + 1), errs
+
+
+@pytest.mark.parametrize("n", [25, 33, 48, 49, 64])
+def test_small_entries_of_a_row(n):
+    """dQ R^-T with R = I returns dQ (Q = 0 leaves the other terms out).  A row is
+    held in 62-bit fixed point against its largest entry (columns relative to
+    their own scale), so an entry 1e-8 of that keeps 2^-62 of it (doubled for
+    the exponents' rounding up, twice) next to its own half ulp."""
+    T = _T()
+    m = 1003
+    dQ = ti.gaussian(m, n, 31)
+    dQ[::3, n - 1] *= 1e-8
+    dQ[1::3, 0] *= 1e-6
+    got = T.backward(_cuda(np.zeros((m, n))), _cuda(np.eye(n)), _cuda(dQ), None).cpu().numpy()
+    col = np.abs(dQ).max(axis=0)
+    row = (np.abs(dQ) / col).max(axis=1)
+    assert np.all(np.abs(got - dQ) <= 2.0 ** -60 * row[:, None] * col + U * np.abs(dQ))
