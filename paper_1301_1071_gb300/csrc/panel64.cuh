@@ -61,7 +61,7 @@ struct Panel64Smem {
     slots = o; o = align_up(o + NS * kPdSlotBytes, 128);
     tiles = o; o += NW * kPdTileBytes;
     r = o; o += static_cast<size_t>(kPdCols * kPdCols) * 8 * NW * (NW + 1) / 2;  // warp q: 8 (q + 1) rows
-    wbuf = o; o += static_cast<size_t>(NW) * 5 * kPdCols * 8;  // two buffers of sums, pivot row, tau, 2 - tau
+    wbuf = o; o += static_cast<size_t>(NW) * 6 * kPdCols * 8;  // two buffers of sums, pivot row, tau, 2 - tau's factors
     total = align_up(o, 16);
   }
 };
@@ -152,8 +152,8 @@ __device__ __forceinline__ long long fixed_of(double x, int sc) {
 }
 
 // One column of the panel factorisation (rows lane + 32 i in a[i]).
-// rbuf: the pivot row (tile 0) is exchanged there, then the factors of 2 - tau;
-// sbuf: the sums.
+// rbuf: the pivot row (tile 0) is exchanged there, then tau and the factors of 2 -
+// tau; sbuf: the sums.
 template <int J>
 __device__ __forceinline__ void panel64_column(double (&a)[kPdRL][kPdCols], double* Rq, double* sbuf, double* rbuf,
                                                int j0, int nb, bool first, int lane) {
@@ -194,9 +194,10 @@ __device__ __forceinline__ void panel64_column(double (&a)[kPdRL][kPdCols], doub
   const double alpha = prow[J], sj = dst[J];
   const Reflector<double> f = make_reflector64(fma(alpha, alpha, sj), alpha);
   const double ps = sj * f.scal;
-  if (lane == 0) {  // the factors of 2 - tau (panel64_tau)
-    rbuf[kPdCols + J] = f.ident ? 2.0 : ps;
-    rbuf[2 * kPdCols + J] = f.ident ? -1.0 : f.ib;
+  if (lane == 0) {  // tau and the factors of 2 - tau (panel64_comp)
+    rbuf[kPdCols + J] = f.tau;
+    rbuf[2 * kPdCols + J] = f.ident ? 2.0 : ps;
+    rbuf[3 * kPdCols + J] = f.ident ? -1.0 : f.ib;
   }
   // lane c: column c's row of R and its coefficient of x.  r' = (alpha r + s) /
   // beta, from tile 1 on as -r + (s + (alpha + beta) r) / beta with alpha + beta
@@ -247,14 +248,11 @@ __device__ __forceinline__ void panel64_factor(double (&a)[kPdRL][kPdCols], doub
 // 2 - tau of the panel's columns, lane c for column c (each of the unit's
 // instructions takes a warp 64 clocks, so one for the eight): s_J / (root
 // (|alpha| + root)) with a relative error of its own -- taken from the rounded
-// tau it errs by tau's rounding, which a block's every tile adds to Q.  rbuf then
-// holds tau and 2 - tau.
-__device__ __forceinline__ void panel64_tau(double* rbuf, int lane) {
-  if (lane < kPdCols) {
-    const double eps = -(rbuf[kPdCols + lane] * rbuf[2 * kPdCols + lane]);
-    rbuf[kPdCols + lane] = 2.0 - eps;
-    rbuf[2 * kPdCols + lane] = eps;
-  }
+// tau it errs by tau's rounding, which a block's every tile adds to Q.  (Nor tau
+// as 2 minus this: d r shares d's rounding with scal = 1 / d; Q's error at 2,000 x 8
+// rose by a tenth.)  Into rbuf's third row.
+__device__ __forceinline__ void panel64_comp(double* rbuf, int lane) {
+  if (lane < kPdCols) rbuf[2 * kPdCols + lane] = -(rbuf[2 * kPdCols + lane] * rbuf[3 * kPdCols + lane]);
   __syncwarp();
 }
 
@@ -299,7 +297,7 @@ __global__ void __launch_bounds__(kPdMaxThreads, 1)
 
   const int j0 = kPdCols * q, nb = n - j0 < kPdCols ? n - j0 : kPdCols;
   double* Rq = reinterpret_cast<double*>(smem + L.r) + kPdCols * kPdCols * q * (q + 1) / 2;
-  double* sbuf = reinterpret_cast<double*>(smem + L.wbuf) + static_cast<size_t>(q) * 5 * kPdCols;
+  double* sbuf = reinterpret_cast<double*>(smem + L.wbuf) + static_cast<size_t>(q) * 6 * kPdCols;
   double* rbuf = sbuf + 2 * kPdCols;
   long long* X = reinterpret_cast<long long*>(smem + L.tiles + static_cast<size_t>(q) * kPdTileBytes);
   double* Xd = reinterpret_cast<double*>(X);
@@ -529,7 +527,7 @@ __global__ void __launch_bounds__(kPdMaxThreads, 1)
       for (int c = 0; c < kPdCols; ++c) a[i][c] = Xd[tile_at(lane + 32 * i, c)];
     panel64_factor<0>(a, Rq, sbuf, rbuf, j0, nb, first, lane);
     __syncwarp();
-    panel64_tau(rbuf, lane);
+    panel64_comp(rbuf, lane);
     // ---- V through the tile: digits (62-bit fixed point per column) and Y
 #pragma unroll
     for (int i = 0; i < RL; ++i)
