@@ -298,7 +298,9 @@ tsqr_status run_tree(const Plan& P, double* R, int64_t ldr, void* work, cudaStre
     const double* C = (l == L - 1) ? ctop : S(l);
     const int64_t cb = (l == L - 1) ? 1 : lv.p;
     // a node is f stacked triangles: the structured product (tree.cu)
-    const cudaError_t e = launch_tree_down(S(l - 1), lv.rows, n, static_cast<int>(lv.b / n), lv.p, T(l), C, cb, st);
+    const int f = static_cast<int>(lv.b / n);
+    const cudaError_t e = launch_tree_down(S(l - 1), lv.rows, n, f, lv.p, T(l), C, cb,
+                                           n >= kTreeCompMinN && tree_up_fits(n, f), st);
     if (e != cudaSuccess) return TSQR_ERR_CUDA;
   }
   return TSQR_OK;

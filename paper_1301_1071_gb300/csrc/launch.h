@@ -33,6 +33,7 @@ cudaError_t launch_form_q(const KernelCfg& k, const void* Y, int64_t m, int n, i
 // the node fits a cluster of f CTAs, one block each (launch_tree_up_cl, same
 // outputs).  Neither: the row-block kernel takes the level.
 constexpr int kTreeClMaxF = 8;  // portable cluster size
+constexpr int kTreeCompMinN = 3;  // comp_at's least n
 bool tree_up_fits(int n, int f);
 cudaError_t launch_tree_up(const double* X, int64_t rows, int n, int f, int64_t p, double* Y, double* Rout,
                            double* Tst, cudaStream_t st);
@@ -43,9 +44,10 @@ cudaError_t launch_tree_up_cl(const double* X, int64_t rows, int n, int f, int64
 // Step-2 down pass of one tree level (binary64): node b's rows of Y (f
 // stacked blocks of n rows, the last node possibly fewer) become its
 // children's coefficient blocks from C (cblocks == 1: one block for all),
-// using Y = [I; V_2; ...; V_f] with V_k upper triangular.
+// using Y = [I; V_2; ...; V_f] with V_k upper triangular.  comp: the T slots
+// hold 1 - tau (launch_tree_up's, n >= kTreeCompMinN).
 cudaError_t launch_tree_down(double* Y, int64_t rows, int n, int f, int64_t p, const double* T, const double* C,
-                             int64_t cblocks, cudaStream_t st);
+                             int64_t cblocks, bool comp, cudaStream_t st);
 
 // Step 3 for binary32 data on the tensor cores (3xTF32), n <= 100; the block
 // and tile geometry (b, B = the Step-1 register tile, bt, kt) of Step 1.  For

@@ -12,8 +12,8 @@
 
 namespace tsqr {
 
-// Where a T slot (n x n, upper triangle) keeps 2 - tau_r (row blocks by panels),
-// in its unused lower triangle, n >= 3.
+// Where a T slot (n x n, upper triangle) keeps 2 - tau_r (row blocks by panels)
+// or 1 - tau_r (tree nodes of k_tree_up), in its unused lower triangle, n >= 3.
 TSQR_HD constexpr int comp_at(int r, int n) { return r + 1 < n ? (r + 1) * n + r : (n - 1) * n; }
 
 TSQR_HD constexpr size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }

@@ -59,10 +59,10 @@ __device__ __forceinline__ void tri_rows(const double* U, const double* D, int l
 // (CJ columns each) forms the panel of one n x n product; KB groups take KB
 // blocks of the node at once (small n: the 24 further blocks of a 25-way node
 // at n = 25 take 3 passes, not 24).  Group 0 forms W.  Threads: KB x group
-// size <= MAXT.
+// size <= MAXT.  comp: T's slots hold 1 - tau (comp_at).
 template <int CJ, int MAXT>
 __global__ void __launch_bounds__(MAXT) k_tree_down(double* Y, int64_t rows, int n, int f, const double* T,
-                                                    const double* C, int64_t cblocks, int KB, int P) {
+                                                    const double* C, int64_t cblocks, int KB, int P, bool comp) {
   extern __shared__ __align__(16) double tsm[];
   const int ncg = (n + CJ - 1) / CJ;
   const int ncp = (ncg + P - 1) / P;  // column groups per panel
@@ -82,19 +82,28 @@ __global__ void __launch_bounds__(MAXT) k_tree_down(double* Y, int64_t rows, int
   const double* Cn = C + (cblocks == 1 ? 0 : node * n * n);
   double* Yn = Y + r0 * n;
   double* B0 = tsm + n * ld;
-  // T (upper triangle; the slot's lower part is not defined) and C, copied
+  const int g = gt / ncp, cg = gt - g * ncp;
+  double tau[2] = {0.0, 0.0}, ca[2] = {1.0, 1.0};  // group 0: tau and 1 - tau of its two rows
+  if (comp && grp == 0) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int r = h == 0 ? g : n - 1 - g;
+      tau[h] = Tn[r * n + r];
+      ca[h] = Tn[comp_at(r, n)];
+    }
+  }
+  // T (upper triangle; with comp the strict one) and C, copied
   // asynchronously (every thread's copies in flight at once; the zeros
   // around them are plain stores)
   for (int idx = tid; idx < n * ld; idx += NT) {
     const int i = idx / ld, c = idx - i * ld;
-    if (c < n && c >= i) cp_async_8(Wb + idx, Tn + i * n + c);
+    if (c < n && c >= i + (comp ? 1 : 0)) cp_async_8(Wb + idx, Tn + i * n + c);
     else Wb[idx] = 0.0;
     if (c < n) cp_async_8(B0 + idx, Cn + i * n + c);
     else B0[idx] = 0.0;
   }
   cp_async_wait_all();
   __syncthreads();
-  const int g = gt / ncp, cg = gt - g * ncp;
   const bool active = grp < KB;  // every thread of a group has a row pair
   // the thread's column group; the last panel may have fewer (or none)
   const bool colok = pnl * ncp + cg < ncg;
@@ -103,19 +112,22 @@ __global__ void __launch_bounds__(MAXT) k_tree_down(double* Y, int64_t rows, int
   // W = T C (group 0, the panel's columns)
   if (grp == 0 && colok) tri_rows<CJ>(Wb, B0, ld, n, g, c0, top, bot);
   __syncthreads();
+  // ... and block 1 of the node, C - W: with comp the strict triangle's sum v
+  // gives W = tau C + v and C - W = (1 - tau) C - v, whose entries are about
+  // 1/sqrt(f) of C's and W's (20,000 x 13 in 157 blocks, two levels: Q's error
+  // 3.3e-16 -> 2.9e-16 with this and the row of R formed as in k_tree_up)
   if (grp == 0 && colok) {
 #pragma unroll
-    for (int b = 0; b < CJ; ++b) {
-      Wb[g * ld + c0 + b] = top[b];
-      if (n - 1 - g != g) Wb[(n - 1 - g) * ld + c0 + b] = bot[b];
+    for (int h = 0; h < 2; ++h) {
+      const int r = h == 0 ? g : n - 1 - g;
+      if (h == 1 && r == g) break;
+#pragma unroll
+      for (int b = 0; b < CJ; ++b) {
+        const double v = h == 0 ? top[b] : bot[b], x = B0[r * ld + c0 + b];
+        Wb[r * ld + c0 + b] = fma(tau[h], x, v);
+        if (c0 + b < cb1) Yn[r * n + c0 + b] = fma(ca[h], x, -v);
+      }
     }
-  }
-  __syncthreads();
-  // block 1 of the node: C - W (the panel's columns)
-  const int pw = cb1 > cb0 ? cb1 - cb0 : 0;
-  for (int idx = tid; idx < n * pw; idx += NT) {
-    const int i = idx / pw, c = cb0 + idx - i * pw;
-    Yn[i * n + c] = B0[i * ld + c] - Wb[i * ld + c];
   }
   // blocks 2..nb: -V_k W, KB at a time (V_k staged whole before its rows
   // are overwritten; the node's other panels stage their own copies before
@@ -175,8 +187,9 @@ __global__ void __launch_bounds__(MAXT) k_tree_down(double* Y, int64_t rows, int
 // = scal x at the end.  Bound by the latency of that chain: with the norm, the
 // scaling and the dots one after the other and the library's root and two
 // divisions in it, a 25-way node at n = 25 took 206 us.
-// The node sits in shared memory, row r at M[r * ldm]; scal_j in the padding
-// column of row j.
+// Row j of R becomes (alpha r + x_j^T a) / beta: r - tau (r + v^T a) would round at
+// r's size.  The node sits in shared memory, row r at M[r * ldm]; scal_j in the
+// padding column of row j, 1 / beta_j in that of row n + j.  (smem: f >= 2 blocks.)
 template <bool WANT_Y>
 __global__ void __launch_bounds__(1024) k_tree_up(const double* X, int64_t rows, int n, int f, double* Y,
                                                   double* Rout, double* Tst, int G) {
@@ -188,7 +201,7 @@ __global__ void __launch_bounds__(1024) k_tree_up(const double* X, int64_t rows,
   const int64_t r0 = node * f * n;
   const int nb = static_cast<int>((rows - r0) / n < f ? (rows - r0) / n : f);
   double* M = usm;                      // nb n rows
-  double* taus = M + nb * n * ldm;      // tau per column
+  double* al = M + nb * n * ldm;        // alpha per column
   const double* Xn = X + r0 * n;
   for (int idx = tid; idx < nb * n * n; idx += NT) {
     const int r = idx / n, cc = idx - r * n;
@@ -231,24 +244,25 @@ __global__ void __launch_bounds__(1024) k_tree_up(const double* X, int64_t rows,
     }
     double s = s0 + s1;
     for (int o = G >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(gmask, s, o);
-    if (c == j) {
+    if (c == j && u == 0) {
       const double alpha = M[j * ldm + j];
       const Reflector<double> f = make_reflector64(fma(alpha, alpha, s), alpha);
-      if (u == 0) {
-        taus[j] = f.tau;
-        M[j * ldm + n] = f.scal;
-        M[j * ldm + j] = f.beta;
-      }
+      al[j] = f.ident ? 1.0 : alpha;  // (a zero column: r' = r)
+      M[j * ldm + n] = f.scal;
+      M[(n + j) * ldm + n] = f.ident ? 1.0 : f.ib;
+      M[j * ldm + j] = f.beta;
     }
     __syncthreads();
-    const double tau = taus[j], scal = M[j * ldm + n];
+    const double scal = M[j * ldm + n];
     if (gram) {
       if (u == 0) Tn[c * n + j] = (M[c * ldm + n] * scal) * s;
-    } else if (live && c > j && tau != 0.0) {
-      // w_c = a_jc + scal x^T a_c; a_c -= (tau w_c scal) x
-      const double tw = tau * fma(scal, s, M[j * ldm + c]);
-      const double tx = tw * scal;
-      if (u == 0) M[j * ldm + c] -= tw;
+    } else if (live && c > j) {
+      // r' = (alpha r + x^T a_c) / beta, a_c -= ((r - r') scal) x
+      const double r = M[j * ldm + c];
+      const double rn = fma(al[j], r, s) * M[(n + j) * ldm + n];
+      const double tx = (r - rn) * scal;
+      __syncwarp(gmask);  // every lane of the group has read r
+      if (u == 0) M[j * ldm + c] = rn;
       double* p = M + (k0 * n + l0) * ldm;
       int lr = l0;
       const int step = (dq * n + dr) * ldm, wrap = (n - len) * ldm;
@@ -277,7 +291,11 @@ __global__ void __launch_bounds__(1024) k_tree_up(const double* X, int64_t rows,
       const int r = idx / n, cc = idx - r * n;
       Yn[idx] = M[r * ldm + cc] * M[cc * ldm + n];
     }
-    for (int i = tid; i < n; i += NT) Tn[i * n + i] = taus[i];
+    for (int i = tid; i < n; i += NT) {
+      const double ca = al[i] * M[(n + i) * ldm + n];  // 1 - tau = alpha / beta
+      Tn[i * n + i] = 1.0 - ca;
+      if (n >= kTreeCompMinN) Tn[comp_at(i, n)] = ca;
+    }
   }
 }
 
@@ -451,7 +469,7 @@ __global__ void __launch_bounds__(1024) k_tree_up_cl(const double* X, int64_t ro
 }  // namespace
 
 cudaError_t launch_tree_down(double* Y, int64_t rows, int n, int f, int64_t p, const double* T, const double* C,
-                             int64_t cblocks, cudaStream_t st) {
+                             int64_t cblocks, bool comp, cudaStream_t st) {
   const int CJ = n > 50 ? 10 : 5;
   const int maxt = CJ == 10 ? 512 : 1024;
   const int ncg = (n + CJ - 1) / CJ;
@@ -486,7 +504,7 @@ cudaError_t launch_tree_down(double* Y, int64_t rows, int n, int f, int64_t p, c
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, fn, Y, rows, n, f, T, C, cblocks, KB, P);
+  return cudaLaunchKernelEx(&cfg, fn, Y, rows, n, f, T, C, cblocks, KB, P, comp);
 }
 
 size_t tree_up_smem(int n, int f) {

@@ -55,3 +55,20 @@ def test_small_entries_of_a_row(n):
     col = np.abs(dQ).max(axis=0)
     row = (np.abs(dQ) / col).max(axis=1)
     assert np.all(np.abs(got - dQ) <= 2.0 ** -60 * row[:, None] * col + U * np.abs(dQ))
+
+
+@pytest.mark.parametrize("m,block_rows,fanout,seeds,bar", [
+    # 157 blocks of 128 rows in two levels of 13; the bar: 5 % above what 63
+    # blocks of 320 rows under one level gave, 2.90e-16 +- 0.02
+    (20_000, 0, 0, 24, 1.05 * 2.90e-16),
+    # 128 blocks in seven levels of 2; the bar: what nodes factored with scaled
+    # vectors and rounded roots and quotients gave, 4.80e-16 +- 0.05
+    (16_384, 128, 2, 12, 4.80e-16),
+])
+def test_tree_levels(m, block_rows, fanout, seeds, bar):
+    """The tree adds no more to Q's error (root mean square over the seeds) than
+    fewer levels, or nodes in plain binary64 steps, did.  (With each level's top
+    block C - W rounded at C's size and rows of R formed as r - tau (r + v^T a)
+    the two were 3.30e-16 and 5.46e-16.)"""
+    errs = [_q_error(ti.gaussian(m, 13, 950 + s), block_rows=block_rows, fanout=fanout) for s in range(seeds)]
+    assert np.sqrt(np.mean(np.square(errs))) <= bar, errs
