@@ -16,6 +16,11 @@ namespace tsqr {
 // or 1 - tau_r (tree nodes of k_tree_up), in its unused lower triangle, n >= 3.
 TSQR_HD constexpr int comp_at(int r, int n) { return r + 1 < n ? (r + 1) * n + r : (n - 1) * n; }
 
+// Tiles of a block of `rows` rows (>= 1): B rows, then bt (<= B) each.  rows + bt
+// can exceed an int's range (blocks have up to 2^31 - 1 rows), rows - B + bt
+// cannot.
+TSQR_HD constexpr int row_tiles(int rows, int B, int bt) { return rows <= B ? 1 : 1 + (rows - B + bt - 1) / bt; }
+
 TSQR_HD constexpr size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // Shared-memory layout of k_local_qr (identical on host and device).

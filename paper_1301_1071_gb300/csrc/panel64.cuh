@@ -288,7 +288,7 @@ __global__ void __launch_bounds__(kPdMaxThreads, 1)
   const int g = lane >> 2, t4 = lane & 3;
   const int64_t row0 = static_cast<int64_t>(blockIdx.x) * b;
   const int rows = static_cast<int>(m - row0 < b ? m - row0 : b);
-  const int ntiles = (rows + TR - 1) / TR;
+  const int ntiles = row_tiles(rows, TR, TR);
   for (int s = threadIdx.x; s < 2 * NS + 1; s += blockDim.x) full[s] = 0;
   // R starts as zero: its entries below the diagonal and of padding columns
   // are read (as part of a column's norm) but never written

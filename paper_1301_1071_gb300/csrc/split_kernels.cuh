@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(kRsThreads, KC <= 2 ? 2 : 1)
   fence_mbar_init();
   const int64_t row0 = static_cast<int64_t>(blockIdx.x) * b;
   const int rows = static_cast<int>(m - row0 < b ? m - row0 : b);
-  const int ntiles = rows <= B ? 1 : 1 + (rows - B + bt - 1) / bt;
+  const int ntiles = row_tiles(rows, B, bt);
   const int ntop = rows < n ? rows : n;
   const int nn = n * n, NT = split_nt(n);
   const double* Cb = Cg + (cblocks == 1 ? 0 : static_cast<int64_t>(blockIdx.x)) * nn;
