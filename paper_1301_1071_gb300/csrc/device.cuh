@@ -9,9 +9,11 @@
 #pragma once
 
 #include <cstdint>
+#include <cstring>
 #include <cuda_runtime.h>
 
 #include "../../include/tsqr.h"
+#include "layout.cuh"
 
 namespace tsqr {
 
@@ -123,27 +125,90 @@ __device__ __forceinline__ void bulk_g2s(void* dst_smem, const void* src_gmem, u
       : "memory");
 }
 
+// Words of a number and back, leading zeros (64 for zero), funnel shift: the
+// intrinsics, and on the host (tests of the integer conversions) plain C++.
+TSQR_HD inline uint32_t hi_word(double x) {
+#ifdef __CUDA_ARCH__
+  return static_cast<uint32_t>(__double2hiint(x));
+#else
+  uint64_t b;
+  std::memcpy(&b, &x, 8);
+  return static_cast<uint32_t>(b >> 32);
+#endif
+}
+TSQR_HD inline uint32_t lo_word(double x) {
+#ifdef __CUDA_ARCH__
+  return static_cast<uint32_t>(__double2loint(x));
+#else
+  uint64_t b;
+  std::memcpy(&b, &x, 8);
+  return static_cast<uint32_t>(b);
+#endif
+}
+TSQR_HD inline double from_words(uint32_t hi, uint32_t lo) {
+#ifdef __CUDA_ARCH__
+  return __hiloint2double(static_cast<int>(hi), static_cast<int>(lo));
+#else
+  const uint64_t b = static_cast<uint64_t>(hi) << 32 | lo;
+  double x;
+  std::memcpy(&x, &b, 8);
+  return x;
+#endif
+}
+TSQR_HD inline uint32_t word_of(float x) {
+#ifdef __CUDA_ARCH__
+  return __float_as_uint(x);
+#else
+  uint32_t b;
+  std::memcpy(&b, &x, 4);
+  return b;
+#endif
+}
+TSQR_HD inline float from_word(uint32_t b) {
+#ifdef __CUDA_ARCH__
+  return __uint_as_float(b);
+#else
+  float x;
+  std::memcpy(&x, &b, 4);
+  return x;
+#endif
+}
+TSQR_HD inline int leading_zeros(unsigned long long u) {
+#ifdef __CUDA_ARCH__
+  return __clzll(static_cast<long long>(u));
+#else
+  return u == 0 ? 64 : __builtin_clzll(u);
+#endif
+}
+TSQR_HD inline uint32_t funnel_right(uint32_t lo, uint32_t hi, int n) {  // 0 < n < 32
+#ifdef __CUDA_ARCH__
+  return __funnelshift_r(lo, hi, n);
+#else
+  return lo >> n | hi << (32 - n);
+#endif
+}
+
 // binary64 <-> binary32, the same results as the conversions, which take 64 clocks
 // a warp on the sub-partition's binary64 unit (idle lanes included): integer
 // operations for zeros and for normal numbers of binary32's range.  4,000,000 x 64
 // binary32: Step 1, which writes T's Gram, 5.24 -> 5.17 ms, the W chain and
 // product of Step 3 0.716 -> 0.680, native Step 3 1.58 -> 1.51.  (Not in
 // k_form_q_tcw, x 100 3.37 -> 3.43 ms, nor in k_build_t, where it changed nothing.)
-__device__ __forceinline__ float f32_of(double x) {
-  const uint32_t hi = static_cast<uint32_t>(__double2hiint(x)), lo = static_cast<uint32_t>(__double2loint(x));
+TSQR_HD inline float f32_of(double x) {
+  const uint32_t hi = hi_word(x), lo = lo_word(x);
   const uint32_t mag = hi & 0x7fffffffu;
   if (mag - 0x38100000u < 0x0fe00000u) {  // 2^-126 <= |x| < 2^128: to nearest, ties to even
     const uint32_t f = ((mag - 0x38000000u) << 3) | (lo >> 29);
-    return __uint_as_float((hi & 0x80000000u) | (f + (((lo & 0x1fffffffu) + 0x0fffffffu + (f & 1u)) >> 29)));
+    return from_word((hi & 0x80000000u) | (f + (((lo & 0x1fffffffu) + 0x0fffffffu + (f & 1u)) >> 29)));
   }
-  if ((mag | lo) == 0) return __uint_as_float(hi);
+  if ((mag | lo) == 0) return from_word(hi);
   return static_cast<float>(x);
 }
-__device__ __forceinline__ double f64_of(float x) {
-  const uint32_t b = __float_as_uint(x), mag = b & 0x7fffffffu;
+TSQR_HD inline double f64_of(float x) {
+  const uint32_t b = word_of(x), mag = b & 0x7fffffffu;
   if (mag - 0x00800000u < 0x7f000000u)  // normal
-    return __hiloint2double(static_cast<int>((b & 0x80000000u) | ((mag >> 3) + 0x38000000u)), static_cast<int>(b << 29));
-  if (mag == 0) return __hiloint2double(static_cast<int>(b), 0);
+    return from_words((b & 0x80000000u) | ((mag >> 3) + 0x38000000u), b << 29);
+  if (mag == 0) return from_words(b, 0);
   return static_cast<double>(x);
 }
 

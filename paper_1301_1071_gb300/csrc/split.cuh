@@ -23,6 +23,7 @@
 // pass through shared memory.
 #pragma once
 
+#include <cmath>
 #include <cstdint>
 
 #include "device.cuh"
@@ -80,13 +81,19 @@ __device__ __forceinline__ int split_int(float acc) {
 
 // P 2^s rounded to nearest (ties up in magnitude) with integer operations;
 // outside the normal range (and for zero) by a call.
-static __device__ __noinline__ double split_to_double_slow(long long P, int s) {
+#ifdef __CUDA_ARCH__
+#define TSQR_SLOW_CALL __noinline__
+#else
+#define TSQR_SLOW_CALL
+#endif
+static TSQR_HD TSQR_SLOW_CALL double split_to_double_slow(long long P, int s) {
   return P == 0 ? 0.0 : ldexp(static_cast<double>(P), s);
 }
-__device__ __forceinline__ double split_to_double(long long P, int s) {
+#undef TSQR_SLOW_CALL
+TSQR_HD inline double split_to_double(long long P, int s) {
   const uint32_t sign = static_cast<uint32_t>(static_cast<unsigned long long>(P) >> 32) & 0x80000000u;
   const unsigned long long u = static_cast<unsigned long long>(P < 0 ? -P : P);
-  const int lz = __clzll(static_cast<long long>(u));
+  const int lz = leading_zeros(u | 1ull);  // at most 63: a shift by 64 has no value
   const unsigned long long w = (u << lz) + 0x400ull;  // bit 63 set; a carry out means 2^64
   // the significand's 53 bits (its hidden bit adds one to the exponent field);
   // a carry out of the rounding leaves w near 0: the exponent takes it
@@ -95,8 +102,8 @@ __device__ __forceinline__ double split_to_double(long long P, int s) {
   const int e = s - lz + (carry ? 1086 : 1085);  // biased exponent less one
   if (static_cast<uint32_t>(e) > 2044u || u == 0ull) return split_to_double_slow(P, s);
   const uint32_t mh = (carry ? 0x100000u : (wh >> 11));
-  const uint32_t ml = __funnelshift_r(wl, wh, 11);
-  return __hiloint2double(static_cast<int>((static_cast<uint32_t>(e) << 20) + mh | sign), static_cast<int>(ml));
+  const uint32_t ml = funnel_right(wl, wh, 11);
+  return from_words(((static_cast<uint32_t>(e) << 20) + mh) | sign, ml);
 }
 
 // sum_D v_D 2^(44 - 8 D), D = 0 .. 7: the digit diagonals of a product of two
