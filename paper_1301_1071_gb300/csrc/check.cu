@@ -25,6 +25,7 @@
 
 #include "../../include/tsqr.h"
 #include "check.h"
+#include "launch.h"
 
 namespace tsqr {
 
@@ -206,14 +207,12 @@ cudaError_t launch_accuracy(int esz, const void* Q, const void* A, const double*
                             double* part, double* out, cudaStream_t st) {
   const AccuracyGeom g = accuracy_geom(m, n);
   if (esz == 8) {
-    cudaError_t e = cudaFuncSetAttribute(k_accuracy<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(g.smem));
+    cudaError_t e = allow_smem(k_accuracy<double>, g.smem);
     if (e != cudaSuccess) return e;
     k_accuracy<double><<<g.grid, kChkThreads, g.smem, st>>>(static_cast<const double*>(Q),
                                                             static_cast<const double*>(A), R, m, n, g.ch, part);
   } else {
-    cudaError_t e = cudaFuncSetAttribute(k_accuracy<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(g.smem));
+    cudaError_t e = allow_smem(k_accuracy<float>, g.smem);
     if (e != cudaSuccess) return e;
     k_accuracy<float><<<g.grid, kChkThreads, g.smem, st>>>(static_cast<const float*>(Q),
                                                            static_cast<const float*>(A), R, m, n, g.ch, part);

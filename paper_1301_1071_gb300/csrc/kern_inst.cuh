@@ -21,7 +21,7 @@ static cudaError_t local_qr_R(const KernelCfg& k, const TSQR_S* A, int64_t m, in
   // the look-ahead form when the tile is one row group
   auto fn = k.NRG == 1 ? k_local_qr<TSQR_S, TSQR_T, NPC, R, MAXT, true>
                        : k_local_qr<TSQR_S, TSQR_T, NPC, R, MAXT, false>;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem_qr);
+  cudaError_t e = allow_smem(fn, k.smem_qr);
   if (e != cudaSuccess) return e;
   fn<<<(unsigned)p, k.NT, k.smem_qr, st>>>(A, m, n, (int)b, (int)bt, kt, k.CS, k.NRG, Y, Rst, Tst, status);
   return cudaGetLastError();
@@ -33,7 +33,7 @@ static cudaError_t form_q_R(const KernelCfg& k, const TSQR_S* Y, int64_t m, int 
                             int32_t* status, cudaStream_t st) {
   if (k.NT > MAXT) return cudaErrorInvalidConfiguration;
   auto fn = k_form_q<TSQR_S, TSQR_T, NPC, R, MAXT>;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem_fq);
+  cudaError_t e = allow_smem(fn, k.smem_fq);
   if (e != cudaSuccess) return e;
   fn<<<(unsigned)p, k.NT, k.smem_fq, st>>>(Y, m, n, (int)b, B, (int)bt, kt, k.fq_rows, k.CS, k.NRG, k.skew, T, C,
                                            cblocks, comp, Q, status);
@@ -83,7 +83,7 @@ static cudaError_t local_r_R(const KernelCfg& k, const TSQR_S* A, int64_t m, int
                              int64_t p, double* Rst, int32_t* status, cudaStream_t st) {
   if (k.NT > MAXT || k.NRG != 1) return cudaErrorInvalidConfiguration;
   auto fn = k_local_qr<TSQR_S, TSQR_T, NPC, R, MAXT, true, false>;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem_qr);
+  cudaError_t e = allow_smem(fn, k.smem_qr);
   if (e != cudaSuccess) return e;
   fn<<<(unsigned)p, k.NT, k.smem_qr, st>>>(A, m, n, (int)b, (int)bt, kt, k.CS, k.NRG, nullptr, Rst, nullptr,
                                            status);
@@ -114,7 +114,7 @@ static cudaError_t local_qr_ng_R(const KernelCfg& k, const TSQR_S* A, int64_t m,
                                  int64_t p, TSQR_S* Y, double* Rst, double* Tst, int32_t* status, cudaStream_t st) {
   if (k.NT > MAXT || k.NRG != 1) return cudaErrorInvalidConfiguration;
   auto fn = k_local_qr<TSQR_S, TSQR_T, NPC, R, MAXT, true, false>;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem_qr);
+  cudaError_t e = allow_smem(fn, k.smem_qr);
   if (e != cudaSuccess) return e;
   fn<<<(unsigned)p, k.NT, k.smem_qr, st>>>(A, m, n, (int)b, (int)bt, kt, k.CS, k.NRG, Y, Rst, Tst, status);
   return cudaGetLastError();
@@ -146,7 +146,7 @@ static cudaError_t rowmul_R(const KernelCfg& k, const TSQR_S* X, const double* M
   if (k.NT > MAXT) return cudaErrorInvalidConfiguration;
   auto fn = k_rowmul<TSQR_S, TSQR_T, NPC, R, MAXT>;
   const size_t smem = k.smem_rm;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(fn, smem);
   if (e != cudaSuccess) return e;
   fn<<<(unsigned)p, k.NT, smem, st>>>(X, M1, Y, M2, m, n, (int)b, k.rm_rows, k.CS, k.NRG, k.skew, out, status);
   return cudaGetLastError();
@@ -178,7 +178,7 @@ cudaError_t TSQR_GRAM_NAME(const void* X, const void* Y, int64_t m, int n, int c
   const size_t smem = 2 * align_up((size_t)chunk * n * sizeof(TSQR_S), 16) + 16;
   auto fn = acc_storage ? (tile == 5 ? k_gram<TSQR_S, 5, TSQR_S> : k_gram<TSQR_S, 4, TSQR_S>)
                         : (tile == 5 ? k_gram<TSQR_S, 5, double> : k_gram<TSQR_S, 4, double>);
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(fn, smem);
   if (e != cudaSuccess) return e;
   fn<<<grid, nt, smem, st>>>(static_cast<const TSQR_S*>(X), static_cast<const TSQR_S*>(Y), m, n, chunk, part,
                              status);

@@ -9,7 +9,7 @@ cudaError_t launch_rowmul_f32_tiles(const float* X, const double* M1, const floa
                                     int n, float* out, cudaStream_t st) {
   const int nin = (X ? 1 : 0) + (Y ? 1 : 0);
   const size_t smem = nin * r32_mat(n) + 2 * r32_tile(n);
-  cudaError_t e = cudaFuncSetAttribute(k_rowmul_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(k_rowmul_f32, smem);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0, per = 1;
   const int nt = kR32Ty * r32_tx(n);
@@ -24,7 +24,7 @@ cudaError_t launch_rowmul_f32_tiles(const float* X, const double* M1, const floa
 cudaError_t launch_form_q_f32_tiles(float* Y, int64_t m, int n, int64_t b, int B, int64_t bt, int kt, int64_t p,
                                     const double* T, const double* C, int64_t cblocks, cudaStream_t st) {
   const size_t smem = 2 * r32_mat(n) + 2 * r32_tile(n);
-  cudaError_t e = cudaFuncSetAttribute(k_form_q_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(k_form_q_f32, smem);
   if (e != cudaSuccess) return e;
   k_form_q_f32<<<(unsigned)p, kR32Ty * r32_tx(n), smem, st>>>(Y, m, n, b, B, (int)bt, kt, T, C, cblocks);
   return cudaGetLastError();

@@ -13,7 +13,7 @@ cudaError_t launch_rowmul_split(const double* X, const double* M, const double* 
             : KC == 2 ? k_rowmul_split<2>
             : KC == 3 ? k_rowmul_split<3>
                       : k_rowmul_split<4>;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  cudaError_t e = allow_smem(fn, smem);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -35,7 +35,7 @@ cudaError_t launch_form_q_split(double* Y, int64_t m, int n, int64_t b, int B, i
             : KC == 2 ? k_form_q_split<2>
             : KC == 3 ? k_form_q_split<3>
                       : k_form_q_split<4>;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  cudaError_t e = allow_smem(fn, smem);
   if (e != cudaSuccess) return e;
   fn<<<static_cast<unsigned>(p), kRsThreads, smem, st>>>(Y, m, n, static_cast<int>(b), B, static_cast<int>(bt), kt, T,
                                                          C, cblocks, comp, status);
@@ -54,7 +54,7 @@ static cudaError_t gram_split(const S* X, const S* Y, int64_t m, int n, double* 
             : n <= 64 ? k_gram_split<S, SYM, TM, 64, SYM ? 3 : 4, 256, 1>
                       : k_gram_split<S, SYM, TM, 32, SYM ? 4 : 7, 416, 1>;
   const size_t smem = GramSplitSmem(n, CR, SYM).total;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  cudaError_t e = allow_smem(fn, smem);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0, per = 1;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;

@@ -15,7 +15,7 @@ cudaError_t launch_form_q_tc(float* Y, int64_t m, int n, int64_t b, int B, int64
     if (cblocks != p) return cudaErrorInvalidValue;  // X_0 goes to each block's own C
     // the W chain (over the T slots and C), then the chunk stream
     const size_t ws = WChainSmem(n).total;
-    cudaError_t e = cudaFuncSetAttribute(k_w_chain, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ws);
+    cudaError_t e = allow_smem(k_w_chain, ws);
     if (e != cudaSuccess) return e;
     k_w_chain<<<static_cast<unsigned>(p), kWcThreads, ws, st>>>(Y, m, n, b, B, static_cast<int>(bt), kt, T, C,
                                                                  cblocks);
@@ -28,7 +28,7 @@ cudaError_t launch_form_q_tc(float* Y, int64_t m, int n, int64_t b, int B, int64
     // staged in 16-row groups 16 bytes apart instead (rows 16-byte aligned)
     auto kern = vw == 4 ? (n % 8 == 0 ? k_form_q_tc<4, true> : k_form_q_tc<4, false>)
                         : (vw == 2 ? k_form_q_tc<2, false> : k_form_q_tc<1, false>);
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -39,7 +39,7 @@ cudaError_t launch_form_q_tc(float* Y, int64_t m, int n, int64_t b, int B, int64
     return cudaGetLastError();
   }
   const size_t smem = FormQTcwSmem(n).total;
-  cudaError_t e = cudaFuncSetAttribute(k_form_q_tcw, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(k_form_q_tcw, smem);
   if (e != cudaSuccess) return e;
   k_form_q_tcw<<<static_cast<unsigned>(p), kTcThreads, smem, st>>>(Y, m, n, static_cast<int>(b), B,
                                                                      static_cast<int>(bt), kt, T, C, cblocks, status);

@@ -8,6 +8,19 @@
 
 namespace tsqr {
 
+// Lets fn be launched with `bytes` of dynamic shared memory.  The attribute
+// belongs to the function, on the whole device: it is set to the same value
+// (the most a CTA can have, less a kernel's few static variables) by every call, so
+// that a host thread never lowers it between another thread's setting and
+// launch.
+constexpr size_t kSmemStatic = 128;
+template <class F>
+inline cudaError_t allow_smem(F* fn, size_t bytes, bool has_static = false) {
+  const size_t most = kSmemMax - (has_static ? kSmemStatic : 0);
+  if (bytes > most) return cudaErrorInvalidValue;
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most));
+}
+
 // Step 1 / tree level: p CTAs, one per row block of b rows (k.kind selects
 // the storage/compute types).
 // Blocks of b rows; a block taller than the register tile (b > k.B) is

@@ -3,6 +3,7 @@
 #include <cfloat>
 
 #include "device.cuh"
+#include "launch.h"
 #include "small.cuh"
 
 namespace tsqr {
@@ -113,7 +114,7 @@ __global__ void k_chol_inv(const double* __restrict__ G, int n, double* __restri
 
 cudaError_t launch_chol_inv(const double* G, int n, double* R, double* Rinv, int32_t* status, cudaStream_t st) {
   const size_t smem = 2 * (size_t)n * n * sizeof(double);
-  cudaError_t e = cudaFuncSetAttribute(k_chol_inv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(k_chol_inv, smem, true);
   if (e != cudaSuccess) return e;
   k_chol_inv<<<1, 128, smem, st>>>(G, n, R, Rinv, status);
   return cudaGetLastError();
@@ -140,7 +141,7 @@ __global__ void k_rinv(const double* __restrict__ R, int64_t ldr, int n, double*
 
 cudaError_t launch_rinv(const double* R, int64_t ldr, int n, double* Rinv, int32_t* status, cudaStream_t st) {
   const size_t smem = 2 * (size_t)n * n * sizeof(double);
-  cudaError_t e = cudaFuncSetAttribute(k_rinv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(k_rinv, smem, true);
   if (e != cudaSuccess) return e;
   k_rinv<<<1, 128, smem, st>>>(R, ldr, n, Rinv, status);
   return cudaGetLastError();
@@ -162,7 +163,7 @@ __global__ void k_tri_mul(const double* __restrict__ R2, const double* R1, int n
 
 cudaError_t launch_tri_mul(const double* R2, const double* R1, int n, double* Rout, int64_t ldr, cudaStream_t st) {
   const size_t smem = (size_t)n * n * sizeof(double);
-  cudaError_t e = cudaFuncSetAttribute(k_tri_mul, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(k_tri_mul, smem, true);
   if (e != cudaSuccess) return e;
   k_tri_mul<<<1, 256, smem, st>>>(R2, R1, n, Rout, ldr);
   return cudaGetLastError();
@@ -229,7 +230,7 @@ __global__ void k_bwd_prep(const double* __restrict__ R, const double* __restric
 cudaError_t launch_bwd_prep(const double* R, const double* dR, const double* G, int n, double* M1, double* M2,
                             int32_t* status, cudaStream_t st) {
   const size_t smem = 3 * (size_t)n * n * sizeof(double);
-  cudaError_t e = cudaFuncSetAttribute(k_bwd_prep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(k_bwd_prep, smem, true);
   if (e != cudaSuccess) return e;
   k_bwd_prep<<<1, 256, smem, st>>>(R, dR, G, n, M1, M2, status);
   return cudaGetLastError();
@@ -457,7 +458,7 @@ __global__ void __cluster_dims__(kJacCl, 1, 1) __launch_bounds__(kJacNT)
 cudaError_t launch_jacobi_svd(const double* R, int64_t ldr, int n, double* Ctop, double* S, double* V,
                               int64_t ldv, int32_t* status, cudaStream_t st) {
   const JacobiSmem L(n);
-  cudaError_t e = cudaFuncSetAttribute(k_jacobi_svd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.bytes);
+  cudaError_t e = allow_smem(k_jacobi_svd, L.bytes, true);
   if (e != cudaSuccess) return e;
   k_jacobi_svd<<<kJacCl, kJacNT, L.bytes, st>>>(R, ldr, n, Ctop, S, V, ldv, status);
   return cudaGetLastError();
@@ -641,7 +642,7 @@ static cudaError_t build_t_typed(double* Tst, int64_t p, int n, int sms, const S
   if (p < 2 * static_cast<int64_t>(sms) || sf.Rout) {
     // few slots: latency decides, so one CTA per slot, a thread per column
     const size_t smem = 2 * static_cast<size_t>(n) * n * sizeof(F);
-    cudaError_t e = cudaFuncSetAttribute(k_build_t_cta<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k_build_t_cta<F>, smem);
     if (e != cudaSuccess) return e;
     k_build_t_cta<F><<<static_cast<unsigned>(p + (sf.Rout ? 1 : 0)), 128, smem, st>>>(Tst, n, sf);
     return cudaGetLastError();
@@ -658,7 +659,7 @@ static cudaError_t build_t_typed(double* Tst, int64_t p, int n, int sms, const S
   const int segs = (n + 31) / 32;
   auto fn = segs == 1 ? k_build_t<F, 1> : segs == 2 ? k_build_t<F, 2> : segs == 3 ? k_build_t<F, 3> : k_build_t<F, 4>;
   if (segs > kBuildTSegs) return cudaErrorInvalidValue;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(fn, smem);
   if (e != cudaSuccess) return e;
   fn<<<static_cast<unsigned>(grid), 32 * warps, smem, st>>>(Tst, p, n);
   return cudaGetLastError();

@@ -490,7 +490,7 @@ cudaError_t launch_tree_down(double* Y, int64_t rows, int n, int f, int64_t p, c
   const int NT = (KB * gsz + 31) / 32 * 32;
   const size_t smem = (1 + KB) * buf;
   auto fn = CJ == 10 ? k_tree_down<10, 512> : k_tree_down<5, 1024>;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(fn, smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(p * P));
@@ -524,7 +524,7 @@ cudaError_t launch_tree_up(const double* X, int64_t rows, int n, int f, int64_t 
   while (G < 32 && G < 2 * (f - 1) && 2 * G * n <= 1024) G *= 2;
   const int NT = (G * n + 31) / 32 * 32;
   auto fn = Y ? k_tree_up<true> : k_tree_up<false>;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(fn, smem);
   if (e != cudaSuccess) return e;
   fn<<<(unsigned)p, NT, smem, st>>>(X, rows, n, f, Y, Rout, Tst, G);
   return cudaGetLastError();
@@ -560,7 +560,7 @@ cudaError_t launch_tree_up_cl(const double* X, int64_t rows, int n, int f, int64
   const int G = tree_up_cl_lanes(n, f);
   const int NT = (G * n + 31) / 32 * 32;
   auto fn = Y ? k_tree_up_cl<true> : k_tree_up_cl<false>;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(fn, smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(p * f));
