@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(kPdMaxThreads, 1)
   const Panel64Smem L(NW, NS);
   uint32_t* full = reinterpret_cast<uint32_t*>(smem + L.cnt);  // passes published
   uint32_t* freed = full + NS;                                  // releases, NW per pass
-  volatile uint32_t* bad = full + 2 * NS;                       // Inf or NaN met in the block
+  uint32_t* bad = full + 2 * NS;  // n less the first column that met Inf or NaN (0: none)
   const int lane = threadIdx.x & 31;
   // Panels differ in work and warp w sits on sub-partition w mod 4 in every CTA:
   // order deals them evenly (choose_panel); with one warp a sub-partition the
@@ -452,7 +452,7 @@ __global__ void __launch_bounds__(kPdMaxThreads, 1)
       // is taken 2^gr smaller and its result shifted back.
       {
         const int s0 = sc + 1023 - biased_exp(w0) - ev[2 * t4], s1 = sc + 1023 - biased_exp(w1) - ev[2 * t4 + 1];
-        int gr = max(0, max(w0 != 0.0 ? -s0 : 0, w1 != 0.0 ? -s1 : 0));
+        int gr = min(max(0, max(w0 != 0.0 ? -s0 : 0, w1 != 0.0 ? -s1 : 0)), 62);  // (a few; more where W' is not finite)
         gr = max(gr, __shfl_xor_sync(0xffffffffu, gr, 1));
         gr = max(gr, __shfl_xor_sync(0xffffffffu, gr, 2));
         const bool grown = __any_sync(0xffffffffu, gr > 0);
@@ -491,7 +491,7 @@ __global__ void __launch_bounds__(kPdMaxThreads, 1)
             const int c = static_cast<int>(bits(7) * 256u + bits(8) - (K2 - 2048u)) >> 12;
             long long r = static_cast<long long>(a) * 1048576 + static_cast<long long>(bb) * 16 + c;
             r += static_cast<long long>(static_cast<unsigned long long>(hi) << 36);
-            if (grown) r <<= gr;
+            if (grown) r *= 1ll << gr;
             X[tile_at(8 * i + 2 * t4 + u, g)] += r;
           }
         }
@@ -509,14 +509,16 @@ __global__ void __launch_bounds__(kPdMaxThreads, 1)
       }
       pos.advance(1, NS);
     }
-    // ---- own panel: fixed point -> binary64, then rows lane + 32 i
+    // ---- own panel: fixed point -> binary64, then rows lane + 32 i.  A column that
+    // met Inf or NaN has no fixed point: NaN, so that its vector, its tau and with
+    // them the block's Q become NaN (a caller that reads Q alone sees it)
     if (q > 0) {
 #pragma unroll 2
       for (int i = 0; i < TR / 8; ++i)
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
           const int k = tile_at(8 * i + 2 * t4 + u, g);
-          Xd[k] = split_to_double(X[k], sc - 1085);
+          Xd[k] = nonfinite ? __longlong_as_double(0x7ff8000000000000ll) : split_to_double(X[k], sc - 1085);
         }
     }
     __syncwarp();
@@ -654,16 +656,16 @@ __global__ void __launch_bounds__(kPdMaxThreads, 1)
       __syncwarp();
     }
   }
-  // ---- R_i (raw signs); a block that met Inf or NaN gives NaN
-  if (__any_sync(0xffffffffu, nonfinite) && lane == 0) *bad = 1;
+  // ---- R_i (raw signs); NaN from the first column that met Inf or NaN on
+  if (nonfinite && t4 == 0) atomicMax(bad, static_cast<unsigned>(n - (j0 + g)));
   __syncthreads();
-  const bool poison = *bad != 0;
+  const int first_bad = n - static_cast<int>(*bad);
   double* Rg = Rst + static_cast<int64_t>(blockIdx.x) * n * n;
   for (int e = lane; e < n * kPdCols; e += 32) {
     const int r = e / kPdCols, c = e - r * kPdCols;
     if (c < nb) {
       double v = (j0 + c >= r && r < rows) ? Rq[r * kPdCols + c] : 0.0;
-      if (poison) v = __longlong_as_double(0x7ff8000000000000ll);
+      if (j0 + c >= first_bad) v = __longlong_as_double(0x7ff8000000000000ll);
       Rg[static_cast<int64_t>(r) * n + j0 + c] = v;
     }
   }
