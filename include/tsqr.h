@@ -158,6 +158,22 @@ tsqr_status tsqr_workspace_size(int32_t op, int64_t m, int64_t n, int32_t dtype,
                                 const tsqr_opts* opts, size_t* bytes);
 
 /*
+ * The least workspace with which `op` runs; tsqr_workspace_size gives what its
+ * fastest form wants.  Below that size (and at least this one) a call takes the
+ * plan that this size is of: FP64 data with n >= 8 is factored column by column
+ * in taller tiles instead of by panels in 128-row tiles (each tile keeps an n x n
+ * T factor in the workspace: 4,000,000 x 64 1,066 MB, 447 MB here), the tree takes
+ * its largest fan-in, and Cholesky QR and the adjoint sum fewer partial Grams.
+ * Results then round differently; tsqr_plan_query and tsqr_launch_count describe
+ * calls with the full size.  The calls that keep R alone (TSQR_OP_R,
+ * TSQR_OP_SVD_VALUES, TSQR_OP_INDIRECT) store no T factors: their fastest form
+ * takes tsqr_workspace_size(TSQR_OP_INDIRECT) bytes (24 MB for those sizes).
+ * Host-only; errors as tsqr_workspace_size.
+ */
+tsqr_status tsqr_workspace_min(int32_t op, int64_t m, int64_t n, int32_t dtype,
+                               const tsqr_opts* opts, size_t* bytes);
+
+/*
  * Direct TSQR (Sec. III-B, with the recursive Step 2 of Sec. III-C, Alg. 2):
  *   Step 1: each row block A_i (block_rows rows, the last one may be short)
  *           is factored by Householder QR, A_i = Q1_i R_i; Q1_i is kept in
@@ -195,7 +211,8 @@ tsqr_status tsqr_svd(const void* A, int64_t m, int64_t n, int64_t lda, int32_t d
  * triangular, diag(R) >= 0) -- the R of tsqr_direct up to rounding.
  * opts->prec: NATIVE or DF64 (FP64 data); TF32X3 only affects Step 3, which
  * this call does not run, and computes as NATIVE.  The workspace is that of
- * TSQR_OP_R (the same size as TSQR_OP_DIRECT).  Errors as tsqr_direct.
+ * TSQR_OP_R (the same size as TSQR_OP_DIRECT; no T factors are kept, so
+ * tsqr_workspace_min is enough).  Errors as tsqr_direct.
  */
 tsqr_status tsqr_r(const void* A, int64_t m, int64_t n, int64_t lda, int32_t dtype,
                    double* R, int64_t ldr,
@@ -259,10 +276,12 @@ tsqr_status tsqr_backward(const void* Q, const double* R, const void* dQ, const 
  * other allocations, a latency-critical caller that cannot pay for the
  * implicit device synchronisation of cudaMalloc/cudaFree, or plain C code
  * without a device allocator.
- *  - Limit: the problem's tsqr_workspace_size(TSQR_OP_DIRECT, ...) must not
- *    exceed TSQR_STATIC_WORK_BYTES (16 MiB; e.g. about 390,000 rows at
- *    n = 25 in FP64 with the default plan); larger problems get
- *    TSQR_ERR_WORKSPACE before any launch.
+ *  - Limit: the problem's tsqr_workspace_min(TSQR_OP_DIRECT, ...) must not
+ *    exceed TSQR_STATIC_WORK_BYTES (16 MiB; about 730,000 rows at n = 25 and
+ *    80,000 at n = 64 in FP64 with the default plan); larger problems get
+ *    TSQR_ERR_WORKSPACE before any launch.  A problem whose
+ *    tsqr_workspace_size is more (n = 64: from 40,000 rows) takes the slower
+ *    plan described there.
  *  - Every GPU that loads the library holds the array until the process exits.
  *  - The first call on each device (with that device current) looks up the
  *    array's device address; make that first call before any stream capture.

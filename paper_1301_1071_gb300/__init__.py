@@ -26,7 +26,7 @@ import threading
 import torch
 
 __all__ = ["direct", "direct_host", "direct_static", "svd", "r", "svd_values", "cholqr", "indirect_refine", "backward", "QRFunction", "TSQRError",
-           "workspace_size", "launch_count", "plan_info", "accuracy", "library_path", "load", "STATUS"]
+           "workspace_size", "workspace_min", "launch_count", "plan_info", "accuracy", "library_path", "load", "STATUS"]
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _LIB_PATH = os.path.join(_HERE, "libtsqr_gb300.so")
@@ -78,6 +78,7 @@ def load():
         OP = ctypes.POINTER(Opts)
         sigs = {
             "tsqr_workspace_size": [I32, I64, I64, I32, OP, ctypes.POINTER(SZ)],
+            "tsqr_workspace_min": [I32, I64, I64, I32, OP, ctypes.POINTER(SZ)],
             "tsqr_direct": [P, I64, I64, I64, I32, P, I64, P, I64, P, SZ, OP, P],
             "tsqr_direct_static": [P, I64, I64, I64, I32, P, I64, P, I64, OP, P],
             "tsqr_direct_host": [P, I64, I64, I32, P, P, P, P, SZ, OP, P, P],
@@ -209,24 +210,45 @@ def _raise(st: int, what: str):
         raise TSQRError(st, what)
 
 
-def workspace_size(op: int, m: int, n: int, dtype: torch.dtype, block_rows=0, fanout=0, prec="native") -> int:
-    lib = load()
+def _workspace_bytes(fn, op, m, n, dtype, block_rows, fanout, prec):
     code = F64 if dtype == torch.float64 else F32
     out = ctypes.c_size_t(0)
     o = _opts(block_rows, fanout, prec=prec)
-    _raise(lib.tsqr_workspace_size(op, m, n, code, ctypes.byref(o), ctypes.byref(out)), "tsqr_workspace_size")
+    _raise(getattr(load(), fn)(op, m, n, code, ctypes.byref(o), ctypes.byref(out)), fn)
     return int(out.value)
+
+
+def workspace_size(op: int, m: int, n: int, dtype: torch.dtype, block_rows=0, fanout=0, prec="native") -> int:
+    """Workspace bytes of a call in its fastest form."""
+    return _workspace_bytes("tsqr_workspace_size", op, m, n, dtype, block_rows, fanout, prec)
+
+
+def workspace_min(op: int, m: int, n: int, dtype: torch.dtype, block_rows=0, fanout=0, prec="native") -> int:
+    """The least workspace a call runs with (in a slower form below
+    ``workspace_size``; see tsqr_workspace_min)."""
+    return _workspace_bytes("tsqr_workspace_min", op, m, n, dtype, block_rows, fanout, prec)
 
 
 def _workspace(op, m, n, dtype, device, block_rows, fanout, work, prec="native"):
     """The caller's workspace when it is a contiguous buffer on ``device`` of
-    at least the bytes the call needs, else a new one."""
-    need = workspace_size(op, m, n, dtype, block_rows, fanout, prec)
+    at least the bytes the call runs with, else a new one: of the bytes its
+    fastest form wants, or, where that much memory is not to be had, of the
+    least."""
     if work is not None and (work.device != torch.device(device) or not work.is_contiguous()):
         raise ValueError(f"work must be a contiguous buffer on {device}, got {work.device}")
-    if work is None or _nbytes(work) < need:
-        work = torch.empty(need, dtype=torch.uint8, device=device)
-    return work
+    # R alone stores no T factors: OP_INDIRECT's R pass is the same (but for df64)
+    sized_as = OP_INDIRECT if op in (OP_R, OP_SVD_VALUES) and prec != "df64" else op
+    need = workspace_size(sized_as, m, n, dtype, block_rows, fanout, prec if sized_as == op else "native")
+    if work is not None and (_nbytes(work) >= need
+                             or _nbytes(work) >= workspace_min(op, m, n, dtype, block_rows, fanout, prec)):
+        return work
+    try:
+        return torch.empty(need, dtype=torch.uint8, device=device)
+    except torch.cuda.OutOfMemoryError:
+        least = workspace_min(op, m, n, dtype, block_rows, fanout, prec)
+        if least >= need:
+            raise
+        return torch.empty(least, dtype=torch.uint8, device=device)
 
 
 def _status(work: torch.Tensor, what: str, check: bool):

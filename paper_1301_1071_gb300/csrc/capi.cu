@@ -52,17 +52,17 @@ cudaError_t launch_rowmul(const KernelCfg& k, const void* X, const double* M1, c
 }
 
 cudaError_t launch_gram(int esz, const void* X, const void* Y, int64_t m, int n, double* part, double* G,
-                        int32_t* status, cudaStream_t st, bool acc_storage, int* colexp) {
+                        int max_parts, int32_t* status, cudaStream_t st, bool acc_storage, int* colexp) {
   const GramGeom g = gram_geom(m, n, esz);
-  int parts = g.grid;
+  int parts = max_parts < g.grid ? max_parts : g.grid;
   const cudaError_t e =
       esz == 8 && n >= kSplitMinN
-          ? launch_gram_split(static_cast<const double*>(X), static_cast<const double*>(Y), m, n, g.grid, &parts, part,
+          ? launch_gram_split(static_cast<const double*>(X), static_cast<const double*>(Y), m, n, parts, &parts, part,
                               colexp, st)
       : esz == 8
           ? launch_gram_f64(X, Y, m, n, g.chunk, g.grid, g.nt, g.tile, acc_storage, part, status, st)
       : !acc_storage && X == Y && n >= kGramSplitF32MinN
-          ? launch_gram_split_f32(static_cast<const float*>(X), m, n, g.grid, &parts, part, st)
+          ? launch_gram_split_f32(static_cast<const float*>(X), m, n, parts, &parts, part, st)
           : launch_gram_f32(X, Y, m, n, g.chunk, g.grid, g.nt, g.tile, acc_storage, part, status, st);
   if (e != cudaSuccess) return e;
   return launch_gram_reduce(part, parts, n, G, status, st);
@@ -541,13 +541,32 @@ tsqr_status run_direct_host(const Plan& P, int chunks, const char* A, char* Qh, 
   return TSQR_OK;
 }
 
+// The plan of `op`.  small: see make_plan.  chunks: the copy chunks of
+// TSQR_OP_DIRECT_HOST (1 elsewhere).
+tsqr_status op_plan(int op, int64_t m, int64_t n, int32_t dtype, const tsqr_opts* o, bool small, Plan* P,
+                    int* chunks) {
+  const int prec = (o && op_takes_prec(op)) ? o->prec : 0, fanout = o ? o->tree_fanout : 0;
+  const int64_t block_rows = o ? o->block_rows : 0;
+  *chunks = 1;
+  const int rc =
+      op == TSQR_OP_DIRECT_HOST
+          ? make_host_plan(m, n, esz_of(dtype), block_rows, fanout, P, chunks, prec, device_sms(), small)
+          : make_plan(m, n, esz_of(dtype), block_rows, fanout, P, prec, device_sms(), small, !op_r_only(op));
+  return static_cast<tsqr_status>(rc);
+}
+
+// ... for a call with this workspace: the fast plan, else (it does not fit) the
+// small one.
 tsqr_status plan_for(int op, int64_t m, int64_t n, int32_t dtype, const tsqr_opts* o, size_t work_bytes,
-                     const void* work, Plan* P) {
-  const int prec = (o && op_takes_prec(op)) ? o->prec : 0;
-  int rc = make_plan(m, n, esz_of(dtype), o ? o->block_rows : 0, o ? o->tree_fanout : 0, P, prec,
-                     device_sms());
-  if (rc != TSQR_OK) return static_cast<tsqr_status>(rc);
-  if (!work || !aligned16(work) || work_bytes < op_bytes(*P, op)) return TSQR_ERR_WORKSPACE;
+                     const void* work, Plan* P, int* chunks = nullptr) {
+  int c = 1;
+  TSQR_TRY(op_plan(op, m, n, dtype, o, false, P, &c));
+  if (!work || !aligned16(work)) return TSQR_ERR_WORKSPACE;
+  if (work_bytes < op_bytes(*P, op)) {
+    TSQR_TRY(op_plan(op, m, n, dtype, o, true, P, &c));
+    if (work_bytes < op_bytes(*P, op)) return TSQR_ERR_WORKSPACE;
+  }
+  if (chunks) *chunks = c;
   return TSQR_OK;
 }
 
@@ -587,15 +606,9 @@ tsqr_status tsqr_launch_count(int32_t op, int64_t m, int64_t n, int32_t dtype, c
     *launches = 2;  // partial sums, ordered combination
     return TSQR_OK;
   }
-  const int prec = (opts && op_takes_prec(op)) ? opts->prec : 0;
   Plan P;
   int chunks = 1;
-  int rc = op == TSQR_OP_DIRECT_HOST
-               ? make_host_plan(m, n, esz, opts ? opts->block_rows : 0, opts ? opts->tree_fanout : 0, &P, &chunks,
-                                prec, device_sms())
-               : make_plan(m, n, esz, opts ? opts->block_rows : 0, opts ? opts->tree_fanout : 0, &P, prec,
-                           device_sms());
-  if (rc != TSQR_OK) return static_cast<tsqr_status>(rc);
+  TSQR_TRY(op_plan(op, m, n, dtype, opts, false, &P, &chunks));
   const int L = static_cast<int>(P.levels.size());
   const int g = P.gram_split ? 1 : 0;               // the T factors' Gram after Step 1
   const int s1 = P.fuse_sign ? 0 : 1;               // the sign fix, where it is a launch of its own
@@ -623,15 +636,9 @@ tsqr_status tsqr_plan_query(int32_t op, int64_t m, int64_t n, int32_t dtype, con
   tsqr_status s = check_opts(opts);
   if (s != TSQR_OK) return s;
   if (op < TSQR_OP_DIRECT || op > TSQR_OP_SVD_VALUES) return TSQR_ERR_ARG;
-  const int prec = (opts && op_takes_prec(op)) ? opts->prec : 0;
   Plan P;
   int chunks = 1;
-  int rc = op == TSQR_OP_DIRECT_HOST
-               ? make_host_plan(m, n, esz, opts ? opts->block_rows : 0, opts ? opts->tree_fanout : 0, &P, &chunks,
-                                prec, device_sms())
-               : make_plan(m, n, esz, opts ? opts->block_rows : 0, opts ? opts->tree_fanout : 0, &P, prec,
-                           device_sms());
-  if (rc != TSQR_OK) return static_cast<tsqr_status>(rc);
+  TSQR_TRY(op_plan(op, m, n, dtype, opts, false, &P, &chunks));
   std::memset(info, 0, sizeof(*info));
   info->block_rows = P.levels[0].b;
   info->blocks = P.levels[0].p;
@@ -667,16 +674,29 @@ tsqr_status tsqr_workspace_size(int32_t op, int64_t m, int64_t n, int32_t dtype,
     return TSQR_OK;
   }
   if (op < TSQR_OP_DIRECT || op > TSQR_OP_SVD_VALUES) return TSQR_ERR_ARG;
-  const int prec = (opts && op_takes_prec(op)) ? opts->prec : 0;
   Plan P;
   int chunks = 1;
-  int rc = op == TSQR_OP_DIRECT_HOST
-               ? make_host_plan(m, n, esz, opts ? opts->block_rows : 0, opts ? opts->tree_fanout : 0, &P, &chunks,
-                                prec, device_sms())
-               : make_plan(m, n, esz, opts ? opts->block_rows : 0, opts ? opts->tree_fanout : 0, &P, prec,
-                           device_sms());
-  if (rc != TSQR_OK) return static_cast<tsqr_status>(rc);
+  TSQR_TRY(op_plan(op, m, n, dtype, opts, false, &P, &chunks));
+  // R alone: the size of tsqr_direct, which a caller may reuse (the call itself
+  // takes less, tsqr_workspace_min)
+  if (op == TSQR_OP_R || op == TSQR_OP_SVD_VALUES)
+    TSQR_TRY(op_plan(TSQR_OP_DIRECT, m, n, dtype, opts, false, &P, &chunks));
   *bytes = op_bytes(P, op);
+  return TSQR_OK;
+}
+
+tsqr_status tsqr_workspace_min(int32_t op, int64_t m, int64_t n, int32_t dtype, const tsqr_opts* opts, size_t* bytes) {
+  size_t most = 0;
+  if (!bytes) return TSQR_ERR_ARG;
+  TSQR_TRY(tsqr_workspace_size(op, m, n, dtype, opts, &most));
+  *bytes = most;
+  if (op == TSQR_OP_ACCURACY) return TSQR_OK;
+  for (const bool small : {false, true}) {
+    Plan P;
+    int chunks = 1;
+    TSQR_TRY(op_plan(op, m, n, dtype, opts, small, &P, &chunks));
+    if (op_bytes(P, op) < *bytes) *bytes = op_bytes(P, op);
+  }
   return TSQR_OK;
 }
 
@@ -690,10 +710,7 @@ tsqr_status tsqr_direct(const void* A, int64_t m, int64_t n, int64_t lda, int32_
   const int esz = esz_of(dtype);
   if (overlaps(A, (size_t)m * n * esz, Q, (size_t)m * n * esz)) return TSQR_ERR_ARG;
   Plan P;
-  int rc = make_plan(m, n, esz, opts ? opts->block_rows : 0, opts ? opts->tree_fanout : 0, &P,
-                     opts ? opts->prec : 0, device_sms());
-  if (rc != TSQR_OK) return static_cast<tsqr_status>(rc);
-  if (!work || work_bytes < P.bytes || !aligned16(work)) return TSQR_ERR_WORKSPACE;
+  TSQR_TRY(plan_for(TSQR_OP_DIRECT, m, n, dtype, opts, work_bytes, work, &P));
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   s = run_direct(P, A, Q, R, ldr, work, st, opts, [](double*, cudaStream_t) { return TSQR_OK; });
   if (s != TSQR_OK) return s;
@@ -713,10 +730,7 @@ tsqr_status tsqr_direct_host(const void* A, int64_t m, int64_t n, int32_t dtype,
   if (overlaps(A, (size_t)m * n * esz, Q, (size_t)m * n * esz)) return TSQR_ERR_ARG;
   Plan P;
   int chunks = 1;
-  int rc = make_host_plan(m, n, esz, opts ? opts->block_rows : 0, opts ? opts->tree_fanout : 0, &P, &chunks,
-                          opts ? opts->prec : 0, device_sms());
-  if (rc != TSQR_OK) return static_cast<tsqr_status>(rc);
-  if (!work || work_bytes < P.bytes || !aligned16(work)) return TSQR_ERR_WORKSPACE;
+  TSQR_TRY(plan_for(TSQR_OP_DIRECT_HOST, m, n, dtype, opts, work_bytes, work, &P, &chunks));
   if (overlaps(dbuf, (size_t)m * n * esz, work, P.bytes)) return TSQR_ERR_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   s = run_direct_host(P, chunks, static_cast<const char*>(A), static_cast<char*>(Q), R, static_cast<char*>(dbuf),
@@ -804,11 +818,11 @@ tsqr_status cholqr(const void* A, int64_t m, int64_t n, int64_t lda, int32_t dty
   const int ni = static_cast<int>(n);
   TSQR_CUDA(cudaMemsetAsync(status, 0, sizeof(int32_t), st));
   // Sec. II-A: A^T A = sum_p A_p^T A_p, Cholesky, then Q = A R^{-1} (Sec. II-C)
-  TSQR_CUDA(launch_gram(esz, A, A, m, ni, part, G, status, st));
+  TSQR_CUDA(launch_gram(esz, A, A, m, ni, part, G, P.gram_grid, status, st));
   TSQR_CUDA(launch_chol_inv(G, ni, R1, Rinv, status, st));
   TSQR_TRY(rowmul(P, A, Rinv, nullptr, nullptr, Q, status, st, R1));
   for (int r = 0; r < refine_steps; ++r) {  // iterative refinement: repeat on the computed Q
-    TSQR_CUDA(launch_gram(esz, Q, Q, m, ni, part, G, status, st));
+    TSQR_CUDA(launch_gram(esz, Q, Q, m, ni, part, G, P.gram_grid, status, st));
     TSQR_CUDA(launch_chol_inv(G, ni, R2, Rinv, status, st));
     TSQR_TRY(rowmul(P, Q, Rinv, nullptr, nullptr, Q, status, st, R2));
     TSQR_CUDA(launch_tri_mul(R2, R1, ni, R1, n, st));
@@ -887,7 +901,7 @@ tsqr_status tsqr_backward(const void* Q, const double* R, const void* dQ, const 
   // G = dQ^T Q; binary64: with the scale of dQ's columns, for the product below
   int* qexp = esz == 8 && dQ && rows_by_digits(n) ? reinterpret_cast<int*>(G + 3 * nn) : nullptr;
   if (qexp) TSQR_CUDA(cudaMemsetAsync(qexp, 0, n * sizeof(int), st));
-  if (dQ) TSQR_CUDA(launch_gram(esz, dQ, Q, m, ni, part, G, status, st, esz == 4, qexp));
+  if (dQ) TSQR_CUDA(launch_gram(esz, dQ, Q, m, ni, part, G, P.gram_grid, status, st, esz == 4, qexp));
   TSQR_CUDA(launch_bwd_prep(R, dR, dQ ? G : nullptr, ni, M1, M2, status, st));
   // dA = (dQ + Q copyltu(M)) R^{-T} = dQ R^{-T} + Q (copyltu(M) R^{-T})
   TSQR_TRY(rowmul(P, dQ, M1, Q, M2, dA, status, st, nullptr, qexp));

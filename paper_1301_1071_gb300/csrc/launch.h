@@ -75,9 +75,10 @@ cudaError_t launch_rowmul(const KernelCfg& k, const void* X, const double* M1, c
 // Partial Grams X^T Y (grid partials of n x n binary64), then their fixed-order sum into G.
 // acc_storage: per-CTA partial Grams accumulate in the storage type (binary32
 // data: the FMA pipe); the cross-CTA sum is always binary64.  binary64 data:
-// launch_gram_split (colexp passed to it).
+// launch_gram_split (colexp passed to it).  max_parts: the partials that part holds.
 cudaError_t launch_gram(int esz, const void* X, const void* Y, int64_t m, int n, double* part, double* G,
-                        int32_t* status, cudaStream_t st, bool acc_storage = false, int* colexp = nullptr);
+                        int max_parts, int32_t* status, cudaStream_t st, bool acc_storage = false,
+                        int* colexp = nullptr);
 
 // binary64 as exact digit products (split_kernels.cuh).  out (+)= X M, n <=
 // kRsMaxN: colsrc / colexp give the scale of X's columns (see k_rowmul_split).
@@ -127,6 +128,6 @@ cudaError_t launch_form_q_f32_tiles(float* Y, int64_t m, int n, int64_t b, int B
 
 // Gram launch geometry shared by the planner and the launcher.
 struct GramGeom { int chunk, grid, nt, tile; };
-GramGeom gram_geom(int64_t m, int n, int esz);
+GramGeom gram_geom(int64_t m, int n, int esz, bool small = false);
 
 }  // namespace tsqr

@@ -162,13 +162,13 @@ PanelCfg choose_panel(int n) {
   return c;  // not reached: one CTA holds at least one slot for every n
 }
 
-GramGeom gram_geom(int64_t m, int n, int esz) {
+GramGeom gram_geom(int64_t m, int n, int esz, bool small) {
   GramGeom g;
   int64_t chunk = (int64_t)(kSmemMax - 64) / (2 * (int64_t)n * esz);
   chunk = chunk > 1024 ? 1024 : chunk;
   chunk = chunk / 16 * 16;
   if (chunk < 16) chunk = 16;
-  const bool digits = esz == 8 && n >= kSplitMinN;
+  const bool digits = esz == 8 && n >= kSplitMinN && !small;
   if (digits) chunk = n <= 64 ? 64 : 32;  // k_gram_split
   g.chunk = (int)chunk;
   const int64_t nchunks = (m + chunk - 1) / chunk;
@@ -181,6 +181,8 @@ GramGeom gram_geom(int64_t m, int n, int esz) {
   g.nt = nt < 256 ? 256 : (nt > 1024 ? 1024 : nt);
   return g;
 }
+
+bool op_r_only(int op) { return op == TSQR_OP_R || op == TSQR_OP_SVD_VALUES || op == TSQR_OP_INDIRECT; }
 
 size_t op_bytes(const Plan& P, int op) {
   return (op == TSQR_OP_CHOLQR || op == TSQR_OP_BACKWARD) ? P.bytes_gram : P.bytes;
@@ -232,7 +234,8 @@ static int64_t panel_block_rows(int64_t m, int64_t f, int64_t slots, int64_t al)
   return rows;
 }
 
-int make_plan(int64_t m, int64_t n, int esz, int64_t block_rows, int fanout, Plan* plan, int prec, int sms) {
+static int plan_form(int64_t m, int64_t n, int esz, int64_t block_rows, int fanout, Plan* plan, int prec, int sms,
+                     bool small, bool t_slots) {
   if (n < 1 || n > TSQR_NMAX || m < n) return TSQR_ERR_SHAPE;
   // every m x n matrix of the call, at 8 bytes an entry, must have a byte
   // size that int64 holds (the planner and the kernels index with it)
@@ -261,7 +264,7 @@ int make_plan(int64_t m, int64_t n, int esz, int64_t block_rows, int fanout, Pla
   // 5.28 (with more, shorter tiles for the T factors and Step 3 to take), 28
   // 7.26 -> 5.88, 32 10.96 -> 5.70, 48 30.9 -> 11.5 (2,000,000 rows 7.64, and 6.31
   // since the panels are dealt evenly)
-  P.panel = kind0 == kKindF64 && n >= kSplitMinN &&
+  P.panel = kind0 == kKindF64 && n >= kSplitMinN && !small &&
             !(n <= 25 && (n + 4) / 5 * 5 + 3 < (n + kPdCols - 1) / kPdCols * kPdCols);
   if (P.panel) P.pq = choose_panel((int)n);
   P.B0 = P.panel ? kPdRows : P.cfg0.B;
@@ -287,7 +290,9 @@ int make_plan(int64_t m, int64_t n, int esz, int64_t block_rows, int fanout, Pla
   const int64_t fmax = P.cfg64.B / n;
   const int ni = static_cast<int>(n);
   int64_t f = fanout;
-  if (fanout <= 0) f = fmax >= kTreeClMaxF && tree_up_fits(ni, 4) ? std::min(fmax, kTreeMaxF) : kTreeClMaxF;
+  if (fanout <= 0)
+    f = small ? (fmax >= 4 && tree_up_fits(ni, 4) ? fmax : kTreeClMaxF)
+              : (fmax >= kTreeClMaxF && tree_up_fits(ni, 4) ? std::min(fmax, kTreeMaxF) : kTreeClMaxF);
   int64_t b0 = block_rows;
   if (b0 <= 0 && P.panel) {
     b0 = panel_block_rows(m, f, (int64_t)(sms < 1 ? kDefaultSMs : sms) * P.ctas0, al);
@@ -309,7 +314,7 @@ int make_plan(int64_t m, int64_t n, int esz, int64_t block_rows, int fanout, Pla
   }
   if (b0 < n) return TSQR_ERR_SHAPE;
   if (b0 > m) b0 = m;  // one block
-  if (fanout <= 0 && tree_up_fits(ni, 4)) {
+  if (fanout <= 0 && !small && tree_up_fits(ni, 4)) {
     auto levels = [&](int64_t g) {
       int l = 0;
       for (int64_t p = (m + b0 - 1) / b0; p > 1; p = (p + g - 1) / g) ++l;
@@ -319,7 +324,7 @@ int make_plan(int64_t m, int64_t n, int esz, int64_t block_rows, int fanout, Pla
     while (f > 2 && levels(f - 1) == l) --f;
   }
   const int64_t kt0 = b0 <= B0 ? 1 : 1 + (b0 - B0 + bt - 1) / bt;
-  // tiles per block: heights up to 2^31 - 1 rows in either form
+  // tiles per block: more of the panel form's short ones, for the heights of the other
   if (kt0 > (P.panel ? 1 << 24 : 1 << 20)) return TSQR_ERR_SHAPE;
   if (f < 2 || (f > fmax && !tree_up_fits(ni, static_cast<int>(f)) && !tree_up_cl_fits(ni, static_cast<int>(f))))
     return TSQR_ERR_SHAPE;
@@ -380,14 +385,14 @@ int make_plan(int64_t m, int64_t n, int esz, int64_t block_rows, int fanout, Pla
     l.off_S = o;
     o = al16_ck(add_ck(o, mul_ck((size_t)l.p, nn, &ok), &ok), &ok);
     l.off_T = o;
-    o = al16_ck(add_ck(o, mul_ck(mul_ck((size_t)l.p, (size_t)l.kt, &ok), nn, &ok), &ok), &ok);
+    if (t_slots) o = al16_ck(add_ck(o, mul_ck(mul_ck((size_t)l.p, (size_t)l.kt, &ok), nn, &ok), &ok), &ok);
   }
   P.off_ctop = o;
   o = al16_ck(add_ck(o, nn, &ok), &ok);
   P.off_small = o;
   o = al16_ck(add_ck(o, kSmallSlots * nn, &ok), &ok);
   P.bytes = o;
-  GramGeom g = gram_geom(m, (int)n, esz);
+  GramGeom g = gram_geom(m, (int)n, esz, small);
   P.gram_chunk = g.chunk;
   P.gram_grid = g.grid;
   P.gram_nt = g.nt;
@@ -402,10 +407,24 @@ int make_plan(int64_t m, int64_t n, int esz, int64_t block_rows, int fanout, Pla
   return TSQR_OK;
 }
 
+int make_plan(int64_t m, int64_t n, int esz, int64_t block_rows, int fanout, Plan* plan, int prec, int sms, bool small,
+              bool t_slots) {
+  int rc = TSQR_ERR_SHAPE;
+  if (!small) rc = plan_form(m, n, esz, block_rows, fanout, plan, prec, sms, false, t_slots);
+  // the sizes that the taller tiles take or refuse (block heights of 2^20 tiles,
+  // 2^31 T slots) are those of either form, so that they do not move with it
+  constexpr int64_t kFarM = int64_t(1) << 24;
+  Plan alt;
+  if (rc == TSQR_ERR_SHAPE) return plan_form(m, n, esz, block_rows, fanout, plan, prec, sms, true, t_slots);
+  if (rc == TSQR_OK && plan->panel && m >= kFarM)
+    rc = plan_form(m, n, esz, block_rows, fanout, &alt, prec, sms, true, t_slots);
+  return rc;
+}
+
 int make_host_plan(int64_t m, int64_t n, int esz, int64_t block_rows, int fanout, Plan* plan, int* chunks,
-                   int prec, int sms) {
+                   int prec, int sms, bool small) {
   Plan P0;
-  int rc = make_plan(m, n, esz, block_rows, fanout, &P0, prec, sms);
+  int rc = make_plan(m, n, esz, block_rows, fanout, &P0, prec, sms, small);
   if (rc != TSQR_OK) return rc;
   if (sms < 1) sms = kDefaultSMs;
   const int64_t slots = (int64_t)sms * P0.ctas0;
@@ -423,7 +442,7 @@ int make_host_plan(int64_t m, int64_t n, int esz, int64_t block_rows, int fanout
       b = (b + al - 1) / al * al;
       if (b >= n && b >= P0.B0) {
         Plan P1;
-        if (make_plan(m, n, esz, b, fanout, &P1, prec, sms) == TSQR_OK) P0 = P1;
+        if (make_plan(m, n, esz, b, fanout, &P1, prec, sms, small) == TSQR_OK) P0 = P1;
       }
     }
   }

@@ -142,8 +142,16 @@ size_t op_bytes(const Plan& P, int op);
 // the Step-1 block height (any value >= n; above the register tile's B rows
 // the block is factored tile by tile); 0 chooses it.
 // `sms` = the device's SM count (sizes the default block height).
+// small: the plan for a workspace that the fast one does not fit -- Step 1 by
+// column-by-column tiles, which are 2.4 (n = 64) to 3.9 (n = 8) times as tall as
+// the panels' 128 rows, so that the T slots take that much less, a tree of the
+// largest fan-in, and at most kMaxGramParts partial Grams.  Also taken where the
+// fast plan's T slots are more than a launch can index.
+// t_slots = false (calls that keep R alone): no T slots.
 int make_plan(int64_t m, int64_t n, int esz, int64_t block_rows, int fanout, Plan* plan, int prec = 0,
-              int sms = kDefaultSMs);
+              int sms = kDefaultSMs, bool small = false, bool t_slots = true);
+// The calls that keep R alone of Step 1.
+bool op_r_only(int op);
 
 // Plan of the host-buffer entry point (tsqr_direct_host): the row blocks are
 // taken in `chunks` (<= kMaxHostChunks) consecutive groups, each a whole
@@ -153,6 +161,6 @@ int make_plan(int64_t m, int64_t n, int esz, int64_t block_rows, int fanout, Pla
 constexpr int kMaxHostChunks = 8;
 constexpr int64_t kHostChunkBytes = 128ll << 20;
 int make_host_plan(int64_t m, int64_t n, int esz, int64_t block_rows, int fanout, Plan* plan, int* chunks,
-                   int prec = 0, int sms = kDefaultSMs);
+                   int prec = 0, int sms = kDefaultSMs, bool small = false);
 
 }  // namespace tsqr

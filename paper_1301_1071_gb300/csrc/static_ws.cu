@@ -44,7 +44,8 @@ extern "C" tsqr_status tsqr_direct_static(const void* A, int64_t m, int64_t n, i
                                           int64_t ldq, double* R, int64_t ldr, const tsqr_opts* opts,
                                           void* stream) {
   size_t need = 0;
-  tsqr_status s = tsqr_workspace_size(TSQR_OP_DIRECT, m, n, dtype, opts, &need);
+  // tsqr_direct takes the small plan where the fast one does not fit
+  tsqr_status s = tsqr_workspace_min(TSQR_OP_DIRECT, m, n, dtype, opts, &need);
   if (s != TSQR_OK) return s;
   if (need > kStaticWorkBytes) return TSQR_ERR_WORKSPACE;  // problem too large for the fixed scratch
   int dev = -1;
