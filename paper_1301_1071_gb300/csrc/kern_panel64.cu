@@ -10,7 +10,7 @@ cudaError_t launch_panel_qr_f64(const PanelCfg& k, const void* A, int64_t m, int
   if (32 * k.NW > kPdMaxThreads) return cudaErrorInvalidConfiguration;
   cudaError_t e = allow_smem(k_panel_qr_f64, k.smem);
   if (e != cudaSuccess) return e;
-  k_panel_qr_f64<<<(unsigned)p, 32 * k.NW, k.smem, st>>>(static_cast<const double*>(A), m, n, (int)b, kt, k.NW, k.NS, k.order,
+  k_panel_qr_f64<<<(unsigned)p, 32 * k.NW, k.smem, st>>>(static_cast<const double*>(A), m, n, (int)b, kt, k.NW, k.NS, k.order, k.sms,
                                                          static_cast<double*>(Y), Rst, Tst, status);
   return cudaGetLastError();
 }

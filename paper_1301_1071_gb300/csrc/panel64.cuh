@@ -268,7 +268,7 @@ __device__ __forceinline__ void panel64_comp(double* rbuf, int lane) {
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kPdMaxThreads, 1)
     k_panel_qr_f64(const double* __restrict__ A, int64_t m, int n, int b, int kt, int NW, int NS, uint64_t order,
-                   double* Y, double* __restrict__ Rst, double* __restrict__ Tst, int32_t* status) {
+                   int sms, double* Y, double* __restrict__ Rst, double* __restrict__ Tst, int32_t* status) {
   constexpr int TR = kPdRows, RL = kPdRL;
   extern __shared__ __align__(128) unsigned char smem[];
   const Panel64Smem L(NW, NS);
@@ -284,7 +284,8 @@ __global__ void __launch_bounds__(kPdMaxThreads, 1)
   // 20.9; 1,000,000 x 72 7.79 and 6.60.)
   const unsigned w = threadIdx.x / 32;
   const int q = NW > 4 ? static_cast<int>((order >> (4 * w)) & 15u)
-                       : static_cast<int>((w + blockIdx.x + blockIdx.x / 152u) % static_cast<unsigned>(NW));
+                       : static_cast<int>((w + blockIdx.x + blockIdx.x / static_cast<unsigned>(sms)) %
+                                         static_cast<unsigned>(NW));
   const int g = lane >> 2, t4 = lane & 3;
   const int64_t row0 = static_cast<int64_t>(blockIdx.x) * b;
   const int rows = static_cast<int>(m - row0 < b ? m - row0 : b);

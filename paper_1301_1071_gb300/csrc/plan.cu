@@ -204,12 +204,12 @@ int resolve_prec(int prec, int esz, int64_t n) {
 // block, 4 levels 2.27 ms, two tiles, 3 levels 1.88; 100,000 x 25: 3 levels
 // 1.19 ms, 2 levels 0.89.  At most kMaxTiles tiles (the rounding of a block's
 // chain grows with them).
-static int64_t panel_block_rows(int64_t m, int64_t f, int64_t slots, int64_t al) {
-  auto levels = [&](int64_t p) {  // in rounds of kDefaultSMs nodes
+static int64_t panel_block_rows(int64_t m, int64_t f, int64_t sms, int64_t slots, int64_t al) {
+  auto levels = [&](int64_t p) {  // in rounds of a node an SM
     int64_t l = 0;
     for (; p > 1;) {
       p = (p + f - 1) / f;
-      l += (p + kDefaultSMs - 1) / kDefaultSMs;
+      l += (p + sms - 1) / sms;
     }
     return l;
   };
@@ -267,6 +267,7 @@ static int plan_form(int64_t m, int64_t n, int esz, int64_t block_rows, int fano
   P.panel = kind0 == kKindF64 && n >= kSplitMinN && !small &&
             !(n <= 25 && (n + 4) / 5 * 5 + 3 < (n + kPdCols - 1) / kPdCols * kPdCols);
   if (P.panel) P.pq = choose_panel((int)n);
+  if (sms > 0) P.pq.sms = sms;
   P.B0 = P.panel ? kPdRows : P.cfg0.B;
   P.ctas0 = P.panel ? P.pq.ctas : P.cfg0.ctas;
   const int64_t B0 = P.B0;
@@ -295,7 +296,7 @@ static int plan_form(int64_t m, int64_t n, int esz, int64_t block_rows, int fano
               : (fmax >= kTreeClMaxF && tree_up_fits(ni, 4) ? std::min(fmax, kTreeMaxF) : kTreeClMaxF);
   int64_t b0 = block_rows;
   if (b0 <= 0 && P.panel) {
-    b0 = panel_block_rows(m, f, (int64_t)(sms < 1 ? kDefaultSMs : sms) * P.ctas0, al);
+    b0 = panel_block_rows(m, f, P.pq.sms, (int64_t)P.pq.sms * P.ctas0, al);
   } else if (b0 <= 0) {
     if (sms < 1) sms = kDefaultSMs;
     const int64_t kmax = kind0 == kKindDF64 ? kMaxTilesDF64 : (kind0 == kKindF32 ? kMaxTilesF32 : kMaxTiles);

@@ -54,10 +54,12 @@ bool choose_cfg(int kind, int n, KernelCfg* out, int64_t want_b = 0, int policy 
 
 // Launch shape of k_panel_qr_f64 (Step 1 of binary64 data): panel warps, ring
 // slots, CTAs per SM, shared memory.
+constexpr int kDefaultSMs = 152;  // GB300
 struct PanelCfg {
   int NW = 0, NS = 0, ctas = 1;
   size_t smem = 0;
   uint64_t order = 0;  // the panel of warp w: bits 4 w .. 4 w + 3
+  int sms = kDefaultSMs;  // the device's SM count
 };
 PanelCfg choose_panel(int n);
 
@@ -121,7 +123,6 @@ constexpr int kMaxTiles = 64;       // binary64 data
 constexpr int kMaxTilesF32 = 128;   // binary32 data: its binary64 tree is costly, its rounding unit large
 constexpr int kMaxTilesDF64 = 8;
 constexpr int64_t kTreeMaxF = 32;  // largest default fan-in of a tree node
-constexpr int kDefaultSMs = 152;  // GB300
 constexpr int kMaxGramParts = 304;   // at most this many partial Grams (2 per SM of a GB300)
 constexpr int kMaxGramParts64 = 608;  // binary64 data (k_gram_split: up to 4 CTAs per SM)
 
