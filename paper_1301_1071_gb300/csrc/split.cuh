@@ -91,8 +91,8 @@ static TSQR_HD TSQR_SLOW_CALL double split_to_double_slow(long long P, int s) {
 }
 #undef TSQR_SLOW_CALL
 TSQR_HD inline double split_to_double(long long P, int s) {
-  const uint32_t sign = static_cast<uint32_t>(static_cast<unsigned long long>(P) >> 32) & 0x80000000u;
-  const unsigned long long u = static_cast<unsigned long long>(P < 0 ? -P : P);
+  const unsigned long long up = static_cast<unsigned long long>(P), u = P < 0 ? 0ull - up : up;
+  const uint32_t sign = static_cast<uint32_t>(up >> 32) & 0x80000000u;
   const int lz = leading_zeros(u | 1ull);  // at most 63: a shift by 64 has no value
   const unsigned long long w = (u << lz) + 0x400ull;  // bit 63 set; a carry out means 2^64
   // the significand's 53 bits (its hidden bit adds one to the exponent field);
@@ -119,11 +119,11 @@ __device__ __forceinline__ long long split_combine(const int (&v)[8], int& rem) 
   return static_cast<long long>(v[0]) * (1ll << 44) + static_cast<long long>(a) * (1ll << 28) +
          static_cast<long long>(b) * (1ll << 12) + c;
 }
-// As P 2^e in units of 2^60: rounded to units of 2^68 (e = 8), cut to 2^60 (e =
-// 0) below 2^54 of those, so that P has at least the 53 bits of its rounding
+// As P 2^e in units of 2^60: cut to those (e = 0) below 2^55 units of 2^68, else
+// rounded to the latter (e = 8), so that P has two bits more than its rounding
 // wherever the operands give them.
 __device__ __forceinline__ long long split_round(long long o, int rem, int& e) {
-  const bool small = static_cast<uint32_t>(static_cast<int>(o >> 32) + 0x400000) < 0x800000u;
+  const bool small = static_cast<uint32_t>(static_cast<int>(o >> 32) + 0x800000) < 0x1000000u;
   e = small ? 0 : 8;
   return small ? o * 256 + (rem >> 4) : o + (rem >> 11);
 }

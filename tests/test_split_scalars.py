@@ -49,7 +49,7 @@ def _nearest(P, s):
 
 def _sums():
     rng = np.random.default_rng(5)
-    P = [0, 1, -1, 2**62, -2**62, 2**63 - 1, -(2**63 - 1), 2**53, 2**53 + 1, 2**54 - 1, 2**54 + 2, -(2**54 + 2),
+    P = [0, 1, -1, 2**62, -2**62, 2**63 - 1, -(2**63 - 1), -2**63, 2**53, 2**53 + 1, 2**54 - 1, 2**54 + 2, -(2**54 + 2),
          2**63 - 2**9, 2**63 - 2**9 - 1, 2**62 + 2**8, 2**62 + 2**8 - 1, 2**62 - 1]
     for k in range(1, 63):
         P += [2**k + 1, -(2**k - 1), int(rng.integers(2**(k - 1), 2**k)), -int(rng.integers(2**(k - 1), 2**k))]
