@@ -448,17 +448,14 @@ __global__ void __launch_bounds__(kPdMaxThreads, 1)
         w0 = fma(2.0, w[0], -w0);
         w1 = fma(2.0, w[1], -w1);
       }
-      // A -= V W': the digits of -W' 2^(ev) relative to the column's scale.  A
-      // column whose W' exceeds twice its norm (tile 0's V_top can grow it)
-      // is taken 2^gr smaller and its result shifted back.
+      // A -= V W': the digits of -W' 2^(ev) relative to the column's scale.  W'_j =
+      // tau_j v_j^T b with b the column after j reflectors, so |W'_j| <= 2 ||b|| / ||v_j||
+      // <= 2 norms, and V's entries are at most 1: the shifts are not negative (but
+      // for a column with Inf or NaN, which is NaN in the end).
       {
         const int s0 = sc + 1023 - biased_exp(w0) - ev[2 * t4], s1 = sc + 1023 - biased_exp(w1) - ev[2 * t4 + 1];
-        int gr = min(max(0, max(w0 != 0.0 ? -s0 : 0, w1 != 0.0 ? -s1 : 0)), 62);  // (a few; more where W' is not finite)
-        gr = max(gr, __shfl_xor_sync(0xffffffffu, gr, 1));
-        gr = max(gr, __shfl_xor_sync(0xffffffffu, gr, 2));
-        const bool grown = __any_sync(0xffffffffu, gr > 0);
         uint32_t h[8];
-        split_digits(split_fixed<62>(-w0, max(s0 + gr, 0)), split_fixed<62>(-w1, max(s1 + gr, 0)), h);
+        split_digits(split_fixed<62>(-w0, max(s0, 0)), split_fixed<62>(-w1, max(s1, 0)), h);
         // matrices 0 .. 3: the eight rows of the four planes
         const uint32_t vl = va + ((lane >> 3) * TR + (lane & 7)) * 16;
 #pragma unroll 2
@@ -469,7 +466,7 @@ __global__ void __launch_bounds__(kPdMaxThreads, 1)
           for (int j = 0; j < 4; ++j) unpack_digits(pk[j], vd[2 * j], vd[2 * j + 1]);
           float acc[5][4];
           // k 0-7: digit v of V against digits s, s + 1 of W'; k 8-15: digit
-          // v + 1 against s - 1, s.  Diagonals 0 .. 9 (dropping from 8 on
+          // v + 1 against s - 1, s.  Diagonals 0 .. 8 (dropping the last too
           // would cost 10 units of the column's fixed point a panel)
 #pragma unroll
           for (int v = 0; v < 8; v += 2)
@@ -492,7 +489,6 @@ __global__ void __launch_bounds__(kPdMaxThreads, 1)
             const int c = static_cast<int>(bits(7) * 256u + bits(8) - (K2 - 2048u)) >> 12;
             long long r = static_cast<long long>(a) * 1048576 + static_cast<long long>(bb) * 16 + c;
             r += static_cast<long long>(static_cast<unsigned long long>(hi) << 36);
-            if (grown) r *= 1ll << gr;
             X[tile_at(8 * i + 2 * t4 + u, g)] += r;
           }
         }
