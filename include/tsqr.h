@@ -80,12 +80,18 @@ typedef enum tsqr_dtype { TSQR_F64 = 0, TSQR_F32 = 1 } tsqr_dtype;
  * tsqr_svd honour it; the Step-2 tree, the SVD of R and all n x n work are
  * binary64 in every mode.
  * NATIVE: the data's type (binary32 with binary32 accumulation for TSQR_F32).
- *         TSQR_F64: binary64 accuracy; from n = 7 on the matrix products of
- *         the tall passes (the trailing updates of Step 1 for most n, T's Gram,
- *         Step 3 for n <= 64) are exact sums of 8-bit digit products on the
- *         tensor cores (Ozaki, Ogita, Oishi, Rump 2012: 54- to 62-bit fixed
- *         point, binary16 operands, exact binary32 sums, one rounding to
- *         binary64), the factorisation of a panel of columns in binary64.
+ *         TSQR_F64: binary64 accuracy in the norm of the operands; from n = 7
+ *         on the matrix products of the tall passes (the trailing updates of
+ *         Step 1 for most n, T's Gram, Step 3 and rows times an n x n matrix for
+ *         n <= 64) are sums of 8-bit digit products on the tensor cores (Ozaki,
+ *         Ogita, Oishi, Rump 2012: binary16 operands, exact binary32 sums, one
+ *         rounding to binary64), the factorisation of a panel of columns in
+ *         binary64.  Fixed point is 62 bits wide: against its column's norm for
+ *         an entry of the tile in Step 1, against its row's (column scales taken
+ *         out) or column's largest entry in the products.  So an entry or a row
+ *         2^-k of that scale keeps 62 - k bits, where binary64 FMAs keep 53: from
+ *         k = 9 on there is less relative accuracy, not normwise: errors of Q, R
+ *         and dA against exact ones are at or below those of binary64 FMA chains.
  * DF64:   TSQR_F64 data only.  Binary64 storage, double-float arithmetic
  *         (pairs of binary32, ~48-bit significand) in Step 1 and Step 3, each
  *         row block scaled by a power of two (exact).  Targets ||Q^TQ - I||
@@ -377,7 +383,8 @@ tsqr_status tsqr_launch_count(int32_t op, int64_t m, int64_t n, int32_t dtype, c
  *   prec            the tsqr_prec the call computes in (TSQR_PREC_AUTO resolved)
  *   step3_tensor    1 when `prec` names a tensor-core form of Step 3 (TF32X3, or
  *                   OZAKI in its range); NATIVE reports 0 also where its
- *                   binary64 products are digit products
+ *                   binary64 products are digit products on the tensor cores
+ *                   (7 <= n <= 64)
  */
 typedef struct tsqr_plan_info {
   int64_t block_rows;

@@ -184,7 +184,9 @@ def launch_count(op: int, m: int, n: int, dtype: torch.dtype, block_rows=0, fano
 def plan_info(op: int, m: int, n: int, dtype: torch.dtype, block_rows=0, fanout=0, prec="native") -> dict:
     """The row-block partition and Step-2 tree a call would use (host-only
     query): block_rows, blocks, tiles_per_block, tree_levels, tree_fanout,
-    the resolved precision and whether Step 3 runs on the tensor cores."""
+    the resolved precision and whether that precision names a tensor-core form
+    of Step 3 (False for "native", also where its products are digit products
+    on the tensor cores).  Describes calls with the full workspace."""
     lib = load()
     code = F64 if dtype == torch.float64 else F32
     info = PlanInfo()
@@ -332,7 +334,7 @@ def _direct_host(A, m, n, dev, block_rows, fanout, out, dbuf, work, copy_stream,
 @_on_device
 def direct_static(A: torch.Tensor, block_rows: int = 0, fanout: int = 0, prec: str = "native"):
     """Direct TSQR on the library's fixed device scratch (no workspace is
-    allocated for the call; problems needing more than 16 MiB of workspace
+    allocated for the call; problems whose ``workspace_min`` exceeds 16 MiB
     are rejected).  Returns (Q, R); synchronises to report device errors."""
     m, n = _check_tall(A)
     A = A.contiguous()

@@ -84,11 +84,8 @@ cudaError_t launch_local_qr(const KernelCfg& k, const void* A, int64_t m, int n,
   }
 }
 
-// Step 1 of direct TSQR: Y_i, R_i and the T slots' tau and Gram entries (the
-// Ozaki form: the Gram entries on the tensor cores after a Step 1 without
-// them).
-// The Householder kernel of Step 1 alone (without its Gram dot products in
-// the Ozaki form).
+// The Householder kernel of Step 1: Y_i, R_i and tau in the T slots, for
+// binary64 arithmetic mostly without T's Gram entries (P.gram_split).
 cudaError_t launch_local_qr_step1(const Plan& P, const void* A, int64_t m, int64_t b, int64_t p, void* Y,
                                   double* Rst, double* Tst, int32_t* status, cudaStream_t st) {
   const Level& l0 = P.levels[0];
@@ -98,6 +95,8 @@ cudaError_t launch_local_qr_step1(const Plan& P, const void* A, int64_t m, int64
                         : launch_local_qr(P.cfg0, A, m, n, b, l0.bt, l0.kt, p, Y, Rst, Tst, status, st);
 }
 
+// Step 1 of direct TSQR: the same, with the Gram entries by a launch of its own
+// where the kernel leaves them out.
 cudaError_t launch_step1(const Plan& P, const void* A, int64_t m, int64_t b, int64_t p, void* Y, double* Rst,
                          double* Tst, int32_t* status, cudaStream_t st) {
   const Level& l0 = P.levels[0];
@@ -322,8 +321,8 @@ tsqr_status run_direct(const Plan& P, const void* A, void* Q, double* R, int64_t
   if (mark(o, 0, st) != TSQR_OK) return TSQR_ERR_CUDA;
   if (launch_local_qr_step1(P, A, P.m, l0.b, l0.p, Q, S(0), T(0), status, st) != cudaSuccess) return TSQR_ERR_CUDA;
   if (mark(o, 1, st) != TSQR_OK) return TSQR_ERR_CUDA;
-  // the T factors' Gram entries on the tensor cores (Ozaki form); like the T
-  // build below, it is part of the Step-2 interval of the stage events
+  // the T factors' Gram entries by digit products; like the T build below, part of
+  // the Step-2 interval of the stage events
   if (P.gram_split && launch_gram_t_split(static_cast<const double*>(Q), P.m, n, l0.b, P.B0, l0.bt, l0.kt, l0.p,
                                           T(0), st) != cudaSuccess)
     return TSQR_ERR_CUDA;

@@ -7,7 +7,8 @@
 // keeps its 128 rows of the current row tile in shared memory as 62-bit
 // fixed-point integers, each column relative to a bound of its whole norm
 // (running R and tile): an orthogonal transformation keeps that norm, so the
-// scale holds for the tile.  Per tile the warp applies the block reflectors I - V_p T_p V_p^T
+// scale holds for the tile.  The accuracy is that of the column (normwise): an
+// entry 2^-k of its column's norm keeps 62 - k bits.  Per tile the warp applies the block reflectors I - V_p T_p V_p^T
 // of the panels p < q as they are published --
 //   W = V_p^T A      digits of A (split from the registers) x digits of V_p,
 //   W' = T_p^T (W + R's rows of panel p)                     in binary64,
@@ -26,8 +27,8 @@
 // fragments.  The running R stays in shared memory: tile t >= 1 factors
 // [R; A_t] with vectors [I; V_t].
 //
-// Measured: Step 1 of 4,000,000 x 64 65.2 -> 20.9 ms plus 3.2 for T's Gram (its
-// bytes 0.6; 2 m n^2 binary64 flops would take 27), 3,000,000 x 32 10.96 -> 5.68.
+// Measured: Step 1 of 4,000,000 x 64 65.2 -> 20.6 ms plus 3.2 for T's Gram (its
+// bytes 0.6; 2 m n^2 binary64 flops would take 27), 3,000,000 x 32 10.96 -> 5.39.
 // Bound by the chain of panels a tile runs through: the binary64 unit is 42 %
 // busy with conversions, the columns and T_p^T.
 #pragma once

@@ -191,8 +191,8 @@ size_t op_bytes(const Plan& P, int op) {
 int resolve_prec(int prec, int esz, int64_t n) {
   if (prec != TSQR_PREC_AUTO) return prec;
   // binary32 data: the Step-3 product on the tensor cores from n = 20 up,
-  // where it outruns the FMA form; binary64 data:
-  // the error-free (Ozaki) tensor-core products where they apply (n <= 32)
+  // where it outruns the FMA form; binary64 data: its one arithmetic, named
+  // OZAKI for n <= 32
   if (esz == 4) return n >= kAutoTf32MinN ? TSQR_PREC_TF32X3 : TSQR_PREC_NATIVE;
   return n <= kOzMaxN ? TSQR_PREC_OZAKI : TSQR_PREC_NATIVE;
 }
@@ -260,10 +260,12 @@ static int plan_form(int64_t m, int64_t n, int esz, int64_t block_rows, int fano
   // binary64 Step 1: panels of 8 columns, or the column-by-column register
   // tile (5 columns a warp) where that pads clearly less.  Step 1 of 3,000,000
   // rows, tile -> panels: n = 8 0.81 -> 0.72 ms, 10 0.87 -> 1.54, 12 1.75 -> 1.67,
-  // 16 3.03 -> 1.88, 17 2.87 -> 3.40, 20 3.19 -> 3.74, 24 5.43 -> 3.85, 25 5.41 ->
-  // 5.28 (with more, shorter tiles for the T factors and Step 3 to take), 28
-  // 7.26 -> 5.88, 32 10.96 -> 5.70, 48 30.9 -> 11.5 (2,000,000 rows 7.64, and 6.31
-  // since the panels are dealt evenly)
+  // 16 3.03 -> 1.88, 17 2.87 -> 3.40, 20 3.19 -> 3.74, 24 5.43 -> 3.85, 28 7.26 ->
+  // 5.88, 32 10.96 -> 5.70, 48 30.9 -> 11.5 (2,000,000 rows 7.64, and 6.33 since the
+  // panels are dealt evenly).  At the line, whole calls of 3,000,000 rows, direct
+  // and R alone, tile / panels: n = 20 4.79 and 3.05 / 6.11 and 3.70, 25 7.61 and
+  // 5.11 / 8.38 and 5.31, 33 15.3 and 10.2 / 14.0 and 7.2, 35 15.8 and 10.5 / 14.6
+  // and 7.6: beyond 25 the tile holds fewer rows and panels win whatever they pad
   P.panel = kind0 == kKindF64 && n >= kSplitMinN && !small &&
             !(n <= 25 && (n + 4) / 5 * 5 + 3 < (n + kPdCols - 1) / kPdCols * kPdCols);
   if (P.panel) P.pq = choose_panel((int)n);

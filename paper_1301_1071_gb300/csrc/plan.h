@@ -130,7 +130,7 @@ constexpr int kMaxGramParts64 = 608;  // binary64 data (k_gram_split: up to 4 CT
 // are returned unchanged): binary32 data at n >= kAutoTf32MinN takes the
 // 3xTF32 Step 3 (measured faster than the binary32 FMA Step 3 from about
 // n = 16 on; below, the chunk stream's per-chunk cost dominates), binary64
-// data at n <= 32 the Ozaki form, everything else the data's own arithmetic.
+// data at n <= 32 OZAKI (native's arithmetic by name), everything else NATIVE.
 constexpr int kAutoTf32MinN = 20;
 // the Ozaki mode's range (above: native)
 constexpr int kOzMaxN = 32;

@@ -671,7 +671,7 @@ cudaError_t launch_build_t(double* Tst, int64_t p, int n, bool binary32, cudaStr
   return binary32 ? build_t_typed<float>(Tst, p, n, sms, sf, st) : build_t_typed<double>(Tst, p, n, sms, sf, st);
 }
 
-// G = sum over the nparts partials, in index order (one thread per entry).
+// G = sum over the nparts partials, in an order that nparts alone fixes.
 constexpr int kGrSlices = 16;
 __global__ void k_gram_reduce(const double* __restrict__ part, int nparts, int n, double* __restrict__ G,
                               int32_t* status) {

@@ -38,7 +38,8 @@ struct SignFix {
 };
 cudaError_t launch_build_t(double* Tst, int64_t p, int n, bool binary32, cudaStream_t st,
                            const SignFix& sf = SignFix());
-// G = sum of the nparts n x n partials in index order (deterministic).
+// G = sum of the nparts n x n partials, in slices of every 16th and those in
+// order (deterministic).
 cudaError_t launch_gram_reduce(const double* part, int nparts, int n, double* G, int32_t* status,
                                cudaStream_t st);
 

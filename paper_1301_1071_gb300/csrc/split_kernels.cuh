@@ -39,10 +39,10 @@ struct RowSplitSmem {
 // columns' largest exponents themselves (split_exp).  add: to what `out` holds.
 // X may be out (each 16-row tile is read before it is written).
 //
-// Bound by the integer unit: per entry about 13 operations to split it and, per
-// output, about 25 to recombine it.  A warp per 16 rows (the fragment's height),
+// Bound by the integer unit: per entry about 14 operations to split it and, per
+// output, about 32 to recombine it.  A warp per 16 rows (the fragment's height),
 // rows by bulk copy one tile ahead.  8,000,000 x 25: 8.02 ms by binary64 FMAs,
-// 2.27 so (its 3.2 GB 0.48); 4,000,000 x 64, two products: 56.1 and 8.6.
+// 2.19 so (its 3.2 GB 0.48); 4,000,000 x 64, two products: 56.1 and 9.0.
 template <int KC>
 __global__ void __launch_bounds__(kRsThreads, KC <= 2 ? 2 : 1)
     k_rowmul_split(const double* X, const double* __restrict__ M, const double* __restrict__ colsrc,
@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(kRsThreads, KC <= 2 ? 2 : 1)
 // Bound by the integer unit (splitting, recombining) and, for n > 32, the
 // tensor products; T X through the binary64 unit would cost more than all rows
 // of a tile (n = 64: 74,000 cycles against 43,000).  1,000,003 x 25: 1.34 ms by
-// binary64 FMAs, 0.46 so (0.4 GB: 0.06); 4,000,000 x 64: 38.9 and 8.0 (4.1 GB: 0.61).
+// binary64 FMAs, 0.48 so (0.4 GB: 0.06); 4,000,000 x 64: 38.9 and 8.7 (4.1 GB: 0.61).
 // ---------------------------------------------------------------------------
 struct FormQSplitSmem {
   size_t b, x, w, cexp, bars, rows, total, buf;
