@@ -107,12 +107,12 @@ cudaError_t launch_step1(const Plan& P, const void* A, int64_t m, int64_t b, int
 }
 
 cudaError_t launch_form_q(const KernelCfg& k, const void* Y, int64_t m, int n, int64_t b, int B, int64_t bt, int kt,
-                          int64_t p, const double* T, const double* C, int64_t cblocks, bool comp, void* Q,
-                          int32_t* status, cudaStream_t st) {
+                          int64_t p, const double* T, const double* C, int64_t cblocks, bool comp, bool rows32,
+                          void* Q, int32_t* status, cudaStream_t st) {
   switch (k.kind) {
     case kKindF64: return launch_form_q_f64(k, Y, m, n, b, B, bt, kt, p, T, C, cblocks, comp, Q, status, st);
     case kKindF32:
-      if (step3_rows32(n) && Y == Q)
+      if (rows32 && Y == Q)
         return launch_form_q_f32_tiles(static_cast<float*>(Q), m, n, b, B, bt, kt, p, T, C, cblocks, st);
       return launch_form_q_f32(k, Y, m, n, b, B, bt, kt, p, T, C, cblocks, comp, Q, status, st);
     case kKindDF64: return launch_form_q_df64(k, Y, m, n, b, B, bt, kt, p, T, C, cblocks, comp, Q, status, st);
@@ -355,7 +355,8 @@ tsqr_status run_direct(const Plan& P, const void* A, void* Q, double* R, int64_t
                                      P.panel, status, st)
       : P.tc3 ? launch_form_q_tc(static_cast<float*>(Q), P.m, n, l0.b, P.B0, l0.bt, l0.kt, l0.p, T(0), C0, cb0,
                                  status, st)
-              : launch_form_q(P.cfg0, Q, P.m, n, l0.b, P.B0, l0.bt, l0.kt, l0.p, T(0), C0, cb0, P.panel, Q, status, st);
+              : launch_form_q(P.cfg0, Q, P.m, n, l0.b, P.B0, l0.bt, l0.kt, l0.p, T(0), C0, cb0, P.panel, P.rows32, Q,
+                              status, st);
   if (e3 != cudaSuccess) return TSQR_ERR_CUDA;
   return mark(o, 3, st);
 }
@@ -399,7 +400,7 @@ tsqr_status rowmul(const Plan& P, const void* X, const double* M1, const void* Y
   const int ni = static_cast<int>(P.n);
   const size_t bytes = static_cast<size_t>(P.m) * P.n * P.esz;
   auto clash = [&](const void* in) { return in && in != out && overlaps(in, bytes, out, bytes); };
-  if (P.esz == 4 && ni >= kRows32MinN && !clash(X) && !clash(Y)) {
+  if (P.esz == 4 && rowmul_rows32(ni) && !clash(X) && !clash(Y)) {
     TSQR_CUDA(launch_rowmul_f32_tiles(static_cast<const float*>(X), M1, static_cast<const float*>(Y), M2, P.m, ni,
                                       static_cast<float*>(out), st));
     return TSQR_OK;
@@ -531,7 +532,7 @@ tsqr_status run_direct_host(const Plan& P, int chunks, const char* A, char* Qh, 
               : P.tc3 ? launch_form_q_tc(reinterpret_cast<float*>(Y), rows, n, l0.b, P.B0, l0.bt, l0.kt, pcnt,
                                          T0 + b0 * l0.kt * nn, Cc, cb, status, st)
                       : launch_form_q(P.cfg0, Y, rows, n, l0.b, P.B0, l0.bt, l0.kt, pcnt, T0 + b0 * l0.kt * nn, Cc, cb, P.panel,
-                                      Y, status, st));
+                                      P.rows32, Y, status, st));
     TSQR_CUDA(cudaEventRecord(ev_q[c], st));
     TSQR_CUDA(cudaStreamWaitEvent(cst, ev_q[c], 0));
     TSQR_CUDA(cudaMemcpyAsync(Qh + r0 * row_bytes, Y, rows * row_bytes, cudaMemcpyDeviceToHost, cst));

@@ -33,10 +33,10 @@ cudaError_t launch_local_qr(const KernelCfg& k, const void* A, int64_t m, int n,
 cudaError_t launch_panel_qr_f64(const PanelCfg& k, const void* A, int64_t m, int n, int64_t b, int kt, int64_t p,
                                 void* Y, double* Rst, double* Tst, int32_t* status, cudaStream_t st);
 // Step 3: p CTAs (B, bt: the tile geometry of Step 1; comp: the T slots hold 2 -
-// tau, comp_at).
+// tau, comp_at; rows32: Plan's).
 cudaError_t launch_form_q(const KernelCfg& k, const void* Y, int64_t m, int n, int64_t b, int B, int64_t bt, int kt,
-                          int64_t p, const double* T, const double* C, int64_t cblocks, bool comp, void* Q,
-                          int32_t* status, cudaStream_t st);
+                          int64_t p, const double* T, const double* C, int64_t cblocks, bool comp, bool rows32,
+                          void* Q, int32_t* status, cudaStream_t st);
 
 // Step-2 up pass of one tree level (binary64): node b = f stacked
 // triangular blocks of X (rows x n) -> its R (raw signs) into Rout's block
@@ -112,15 +112,29 @@ cudaError_t launch_gram_split_f32(const float* X, int64_t m, int n, int max_part
 cudaError_t launch_gram_t_split(const double* Y, int64_t m, int n, int64_t b, int B, int64_t bt, int kt, int64_t p,
                                 double* T, cudaStream_t st);
 
-// binary32 row products in 128-row tiles (rows32.cuh), n >= kRows32MinN:
-// out = X M1 + Y M2 (either input NULL; out may be an input), and Step 3 in
-// binary32 arithmetic (Q over Y).  Below n = 8 a thread's 8 columns are padding
-// in part (4,000,000 x 8, Step 1, 3 and adjoint: 1.37 -> 1.15 ms).  Step 3 with
-// odd n > 64 keeps k_form_q: rows copied 4 bytes at a time, and two tiles and
-// two matrices leave one CTA an SM (2,000,000 x 77 with adjoint 16.5 ms there,
-// 16.8 here; x 98 27.2 there, 25.0 here).
+// binary32 row products in 128-row tiles (rows32.cuh): out = X M1 + Y M2 (either
+// input NULL; out may be an input), and Step 3 in binary32 arithmetic (Q over Y).
+// Rows times a matrix, GB300, the earlier kernel / this: n = 8 at 300,000 rows 1.43,
+// n = 13 .. 61 odd 0.93 to 1.25, n = 64 1.39 to 1.65; but rows of odd length are
+// copied 4 bytes at a time, and above n = 64 one CTA an SM is left: 1,500,000 x 69
+// 0.78, 77 0.85, 81 0.99, 89 1.08: odd n from 65 to 80 keep k_rowmul.
 constexpr int kRows32MinN = 8;
-constexpr bool step3_rows32(int n) { return n >= kRows32MinN && (n <= 64 || n % 2 == 0); }
+constexpr bool rowmul_rows32(int64_t n) { return n >= kRows32MinN && (n <= 64 || n > 80 || n % 2 == 0); }
+// Step 3 of p row blocks: a CTA has 16 ceil(n / 8) threads here, 128 and more in
+// k_form_q, so narrow matrices need several CTAs an SM to gain.  k_form_q's time
+// over this, blocks of 1,024 rows or the planner's: n = 52 .. 64 1.03 to 3.9 at any
+// p; n = 33 .. 50 0.66 to 0.97 at 1 .. 147 blocks, 1.12 to 2.2 from 293 on; n = 16 ..
+// 29 0.5 to 1.0 up to 293 blocks, 0.94 to 2.06 at 586 and more; n = 8 .. 15 0.5 to
+// 1.0 at 608 (tall ones too), from 1,465 on 1.1 to 1.9 but for 13 and 15 (0.91,
+// 0.94).  Odd n > 64 as above (2,000,000 x 77 with adjoint 16.5 ms in k_form_q, 16.8
+// here), even ones 1.02 to 1.6 at any p.
+constexpr bool step3_rows32(int n, int64_t p, int64_t sms) {
+  return n < kRows32MinN || (n > 64 && n % 2) ? false
+         : n >= 52                            ? true
+         : n >= 32                            ? 4 * p >= 7 * sms
+         : n >= 16                            ? p >= 3 * sms
+                                              : p >= 8 * sms && !(n >= 13 && n % 2);
+}
 cudaError_t launch_rowmul_f32_tiles(const float* X, const double* M1, const float* Y, const double* M2, int64_t m,
                                     int n, float* out, cudaStream_t st);
 cudaError_t launch_form_q_f32_tiles(float* Y, int64_t m, int n, int64_t b, int B, int64_t bt, int kt, int64_t p,

@@ -340,6 +340,7 @@ static int plan_form(int64_t m, int64_t n, int esz, int64_t block_rows, int fano
   P.split3 = kind0 == kKindF64 && rows_by_digits(n);
   P.gram_split = kind0 == kKindF64 && n >= kSplitMinN && (P.panel || P.cfg0.NRG == 1);
   P.fuse_sign = P.gram_split && !P.oz3;
+  P.rows32 = esz == 4 && step3_rows32((int)n, (m + b0 - 1) / b0, P.pq.sms);
   {
     const int kind_rm = esz == 4 ? kKindF32 : kKindF64;
     // the coefficient blocks' padded width: the wider of the two tile widths'

@@ -93,6 +93,7 @@ struct Plan {
   // kRowSplitMaxN), and Step 1 without its Gram dot products, the T factors'
   // Gram by digit products (k_gram_split; one-row-group tiles)
   bool split3 = false, gram_split = false;
+  bool rows32 = false;  // binary32 arithmetic: Step 3 in 128-row pieces (k_form_q_f32)
   // the sign fix of the top R rides in the top level's T build (one launch
   // less; the explicit Ozaki form keeps its own launch for it)
   bool fuse_sign = false;
