@@ -124,6 +124,7 @@ constexpr int kMaxTiles = 64;       // binary64 data
 constexpr int kMaxTilesF32 = 128;   // binary32 data: its binary64 tree is costly, its rounding unit large
 constexpr int kMaxTilesDF64 = 8;
 constexpr int64_t kTreeMaxF = 32;  // largest default fan-in of a tree node
+constexpr int64_t kTreeNarrowN = 16, kTreeOneLevelF = 80;  // ... of a single level of triangles n <= 16
 constexpr int kMaxGramParts = 304;   // at most this many partial Grams (2 per SM of a GB300)
 constexpr int kMaxGramParts64 = 608;  // binary64 data (k_gram_split: up to 4 CTAs per SM)
 

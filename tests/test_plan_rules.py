@@ -17,6 +17,14 @@ def _T():
     return T
 
 
+@pytest.mark.parametrize("m,n,dt,levels", [(40_000, 8, torch.float32, 1), (40_000, 3, torch.float64, 1),
+                                           (40_000, 20, torch.float64, 2), (600_000, 8, torch.float64, 2)])
+def test_one_level_of_narrow_triangles(m, n, dt, levels):
+    T = _T()
+    info = T.plan_info(T.OP_DIRECT, m, n, dt)
+    assert info["tree_levels"] == levels and (levels > 1 or info["blocks"] == info["tree_fanout"])
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("m,n,dt", [
     (10_000, 11, torch.float64), (3_000, 92, torch.float64), (130, 65, torch.float64), (40_000, 50, torch.float64),
