@@ -416,6 +416,25 @@ static int plan_form(int64_t m, int64_t n, int esz, int64_t block_rows, int fano
   return TSQR_OK;
 }
 
+// Whether the tiles of the small plan S take less time than the panels of F, by
+// the chain that one CTA and the tree run through, in n us.  Few blocks (at most
+// one an SM): a tile of 320 or 512 rows in one CTA against two to five panel
+// tiles, which the panel plan joins to save a tree level.  A panel tile takes
+// 4.4 the first (n = 16 .. 64: 62, 99, 141, 194, 308 us at 16, 22, 32, 40, 64), 3.2
+// each further one, with Step 3 by FMAs (n > 64) 10; a column tile of R rows a
+// thread 0.28 R + 0.2 + 0.065 n (n = 11, 32, 50, 64: 40, 219, 300, 530); a level 5 to
+// 8.5 (up, T, down).  10,000 x 11: panels 232 us, tiles 163; 40,000 x 50 2.11 ms and
+// 1.63; 3,000 x 92 4.93 and 3.70; 130 x 65 1.10 and 0.76; 10,000 x 64 panels 1.82, tiles
+// 2.12.
+static bool tiles_faster(const Plan& F, const Plan& S, int64_t sms) {
+  const Level &a = F.levels[0], &b = S.levels[0];
+  if (a.kt < 2 || b.kt != 1 || b.p > sms) return false;
+  const double n = (double)F.n, level = 5.0 + 0.14 * std::min(n, 25.0);
+  const double panel = (4.4 + (F.n <= kRowSplitMaxN ? 3.2 : 10.0) * (a.kt - 1)) * (kPdCols * F.pq.NW / n);
+  const double tile = 1.12 * (0.28 * S.cfg0.R + 0.2 + 0.065 * n);
+  return tile + level * (double)(S.levels.size() - 1) < panel + level * (double)(F.levels.size() - 1);
+}
+
 int make_plan(int64_t m, int64_t n, int esz, int64_t block_rows, int fanout, Plan* plan, int prec, int sms, bool small,
               bool t_slots) {
   int rc = TSQR_ERR_SHAPE;
@@ -427,6 +446,10 @@ int make_plan(int64_t m, int64_t n, int esz, int64_t block_rows, int fanout, Pla
   if (rc == TSQR_ERR_SHAPE) return plan_form(m, n, esz, block_rows, fanout, plan, prec, sms, true, t_slots);
   if (rc == TSQR_OK && plan->panel && m >= kFarM)
     rc = plan_form(m, n, esz, block_rows, fanout, &alt, prec, sms, true, t_slots);
+  else if (rc == TSQR_OK && plan->panel && block_rows <= 0 && plan->levels[0].kt > 1 &&
+           plan_form(m, n, esz, block_rows, fanout, &alt, prec, sms, true, t_slots) == TSQR_OK &&
+           tiles_faster(*plan, alt, plan->pq.sms))
+    *plan = alt;
   return rc;
 }
 

@@ -17,6 +17,16 @@ def _T():
     return T
 
 
+@pytest.mark.parametrize("m,n,tiles", [
+    (10_000, 11, 1), (10_000, 16, 1), (3_000, 92, 1), (130, 65, 1), (40_000, 50, 1),  # register tiles
+    (10_000, 64, 2), (150_000, 48, 4), (400_000, 64, 11),                              # panels of 128 rows
+])
+def test_panels_or_tiles(m, n, tiles):
+    T = _T()
+    for op in (T.OP_DIRECT, T.OP_R, T.OP_SVD):  # the same plan, so that R is the same
+        assert T.plan_info(op, m, n, torch.float64)["tiles_per_block"] == tiles
+
+
 @pytest.mark.parametrize("m,n,dt,levels", [(40_000, 8, torch.float32, 1), (40_000, 3, torch.float64, 1),
                                            (40_000, 20, torch.float64, 2), (600_000, 8, torch.float64, 2)])
 def test_one_level_of_narrow_triangles(m, n, dt, levels):

@@ -78,7 +78,7 @@ def test_binding_workspace(monkeypatch):
     """The binding keeps a buffer the call runs with, and takes the least one where
     the full size cannot be allocated (on the CPU allocator here)."""
     T = _T()
-    m, n = 40_000, 64
+    m, n = 400_000, 64
     full, least = (f(T.OP_DIRECT, m, n, torch.float64) for f in (T.workspace_size, T.workspace_min))
     assert least < full
 
