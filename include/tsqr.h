@@ -91,7 +91,8 @@ typedef enum tsqr_dtype { TSQR_F64 = 0, TSQR_F32 = 1 } tsqr_dtype;
  *         out) or column's largest entry in the products.  So an entry or a row
  *         2^-k of that scale keeps 62 - k bits, where binary64 FMAs keep 53: from
  *         k = 9 on there is less relative accuracy, not normwise: errors of Q, R
- *         and dA against exact ones are at or below those of binary64 FMA chains.
+ *         and dA against exact ones measure up to half below those of binary64
+ *         FMA chains (at most a tenth above, 2,000 x 8 at kappa 1e4).
  * DF64:   TSQR_F64 data only.  Binary64 storage, double-float arithmetic
  *         (pairs of binary32, ~48-bit significand) in Step 1 and Step 3, each
  *         row block scaled by a power of two (exact).  Targets ||Q^TQ - I||
