@@ -138,8 +138,8 @@ typedef struct tsqr_opts {
                           cluster of f CTAs, one R factor each), else
                           TSQR_ERR_SHAPE.  Automatic: one CTA per node with
                           as many R factors as the binary64 register tile has
-                          rows for, at most 32 and no more than the number of
-                          levels needs, where that is at least 8 and 4 fit the
+                          rows for, at most 32 (80 where one level of n <= 16
+                          takes them) and no more than the number of levels needs, where that is at least 8 and 4 fit the
                           CTA; else 8 per node (on a cluster where one CTA
                           does not hold them). */
   int32_t sync;        /* 1 = synchronise the stream and return the device status */
@@ -167,7 +167,7 @@ tsqr_status tsqr_workspace_size(int32_t op, int64_t m, int64_t n, int32_t dtype,
 /*
  * The least workspace with which `op` runs; tsqr_workspace_size gives what its
  * fastest form wants.  Below that size (and at least this one) a call takes the
- * plan that this size is of: FP64 data with n >= 8 is factored column by column
+ * plan that this size is of: FP64 data with n >= 7 is factored column by column
  * in taller tiles instead of by panels in 128-row tiles (each tile keeps an n x n
  * T factor in the workspace: 4,000,000 x 64 1,066 MB, 447 MB here), the tree takes
  * its largest fan-in, and Cholesky QR and the adjoint sum fewer partial Grams.
